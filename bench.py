@@ -151,15 +151,15 @@ def offdiag_nnz_per_free_row(m) -> float:
 
 
 def kernel_source_hash() -> str:
-    """Hash of the PCG kernels' source: solve.cu, common.cuh and the lines of
+    """Hash of the PCG kernels' source: team.cu, cg.cuh, common.cuh and the lines of
     kernels.h that concern the PCG (its constants and launchers)."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2203_02054_gb300", "csrc")
-    for f in ("solve.cu", "common.cuh"):
+    for f in ("team.cu", "cg.cuh", "common.cuh"):
         with open(os.path.join(csrc, f), "rb") as fh:
             h.update(fh.read())
     with open(os.path.join(csrc, "kernels.h")) as fh:
-        h.update("".join(line for line in fh if "PCG_" in line or "pcg" in line).encode())
+        h.update("".join(line for line in fh if "TEAM_" in line or "team" in line).encode())
     return h.hexdigest()[:16]
 
 
@@ -545,10 +545,9 @@ def main():
     units = float(m.n_tets) * n_iters * args.steps * world
     value, ms_max = aggregate(ms, float(m.n_tets) * n_iters * args.steps, pg, "cuda")
     stats = casim.casim_get_stats(sim.h)
-    # 2 hash binning + 1 single-pass scan + narrow phase + spring update + ray casts + local step + PCG; the
-    # dataflow PCG (kernel 5) forms the right-hand side and finalizes the iteration itself, the others need 2
-    # launches more
-    kernels_per_iter = 8 if stats.pcg_kernel == 5 else 10
+    # 2 hash binning + 1 single-pass scan + narrow phase + spring update + ray casts + local step + RHS gather + PCG; the
+    # team PCG (kernel 5) finalizes the iteration itself, the others need 1 launch more
+    kernels_per_iter = 9 if stats.pcg_kernel == 5 else 10
     gpu_launches = kernels_per_iter * n_iters * args.steps
     hist = casim.casim_get_history(sim.h, n_iters)
 
@@ -600,8 +599,7 @@ def main():
             "gpu_launches": gpu_launches,
             "roofline": {"bound": "hbm", "kernel": {1: "k_pcg (streaming)", 2: "k_pcg_rr (register-resident)",
                                                     3: "k_pcg_cluster", 4: "k_pcg_seg (segmented)",
-                                                    5: "k_pcg_df (dataflow, register-resident, two-level "
-                                                       "preconditioner)"}
+                                                    5: "k_pcg_team (vectors on chip, two-level preconditioner)"}
                          .get(stats.pcg_kernel, "k_pcg"),
                          "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                          "peak_kind": peak_kind, "traffic": recorded_traffic("k_pcg"),

@@ -88,37 +88,39 @@ typedef struct {
   uint64_t wait_budget_cycles;  /* SM clock cycles a grid-barrier wait may spin
                                    before the kernel gives up with CASIM_E_TIMEOUT;
                                    0 selects the default (about 2 s)                 */
-  int32_t pcg_kernel;       /* PCG kernel: 0 auto (one robot: MIXED 5 if it fits,
-                               else 2 if it fits, else 1; several robots: 4 if it
-                               fits, else 3, else 1);
+  int32_t pcg_kernel;       /* PCG kernel: 0 auto (5 if it fits, else for one robot
+                               2 if it fits, else 1; for several 4 if it fits,
+                               else 3, else 1);
                                1 streaming (whole grid, vectors in memory, any
                                size); 2 register-resident (whole grid, one row per
                                thread, grid barriers); 3 cluster (one 16-CTA
                                cluster per robot, vectors in shared memory, robots
                                from a work queue); 4 segmented streaming (blocks
                                assigned to robots, one CG per robot, shared grid
-                               barriers); 5 dataflow (MIXED only: register-resident
-                               without grid barriers; every shared value carries
-                               its CG epoch and readers wait for the rows they
-                               read).
+                               barriers); 5 team (vectors on chip; the blocks of a
+                               robot form a team that exchanges tagged words and
+                               waits only for one another; chosen automatically in
+                               both precisions, with one robot or several, up to
+                               about 230,000 free vertices per robot in MIXED and
+                               58,000 in FP64; forced, it is accepted in MIXED up
+                               to 384 free vertices per SM).
                                A forced kernel that does not fit gives
                                CASIM_E_INVALID at upload                           */
   int32_t debug_flags;      /* test-only fault injection, 0 in normal use:
                                CASIM_DEBUG_BARRIER_NEVER_COMPLETES makes the PCG
-                               grid barrier (kernels 1, 2 and 4) or the partial
-                               poll (kernel 5) wait for one block more than it
-                               has (the cluster kernel uses the hardware cluster
+                               grid barrier (kernels 1, 2 and 4) or the teams'
+                               rounds (kernel 5) wait for one block more than they
+                               have (the cluster kernel uses the hardware cluster
                                barrier), so every wait runs out of
                                wait_budget_cycles and the step ends with
                                CASIM_E_TIMEOUT; CASIM_DEBUG_CORRUPT_INCIDENCE
                                (checked builds only, else CASIM_E_INVALID) plants
                                an out-of-range gather index                      */
-  int32_t pcg_precond;      /* preconditioner of the dataflow kernel (5): 0 auto =
-                               two-level (Jacobi plus an additive coarse
-                               correction over aggregates of a third of a block,
-                               Galerkin
-                               coarse matrix of the Laplacian, its inverse formed
-                               at upload); 1 Jacobi only.  Other kernels use
+  int32_t pcg_precond;      /* preconditioner of the team (5) and segmented (4)
+                               kernels: 0 auto = two-level (Jacobi plus an additive
+                               coarse correction, Galerkin coarse matrix of the
+                               Laplacian, its inverse formed at upload; kernel 4
+                               in MIXED only); 1 Jacobi only.  Other kernels use
                                Jacobi                                            */
   int32_t broad_phase;      /* collision broad phase: 0 spatial hash rebuilt every
                                iteration; 1 AABB trees (Sec. II-B) over the tets
@@ -132,10 +134,9 @@ typedef struct {
                                one warp per query vertex).  Results do not depend
                                on them except for the summation order of the
                                energy statistic; the autotuner picks them        */
-  int32_t pcg_block;        /* rows (threads) per block of the dataflow PCG (5): 0
-                               auto = 288 (9 warps; aggregates of 96 rows) when the
-                               system fits one such block per SM, else 384
-                               (aggregates of 128); 288 or 384 forces it          */
+  int32_t pcg_block;        /* free vertices per block of the team PCG (5) in MIXED:
+                               0 auto (the shortest blocks that one wave of the
+                               SMs holds, at least 96); 288 or 384 forces it      */
 } casim_params;
 
 #define CASIM_DEBUG_BARRIER_NEVER_COMPLETES 1

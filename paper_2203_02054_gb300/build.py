@@ -21,7 +21,7 @@ BUILD_CHECKED = os.path.join(HERE, "_build", "checked")
 LIB = os.path.join(HERE, "libcasim.so")
 LIB_CHECKED = os.path.join(HERE, "libcasim_checked.so")
 
-SOURCES = ["api.cu", "collision.cu", "solve.cu", "adjoint.cu", "noalloc.cu", "remesh.cu", "anderson.cu"]
+SOURCES = ["api.cu", "collision.cu", "solve.cu", "team.cu", "adjoint.cu", "noalloc.cu", "remesh.cu", "anderson.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-I", CSRC, "-I", INCLUDE]

@@ -475,6 +475,7 @@ __global__ void k_adj_diag_springs(Dev<T> d, AdjDev<T> a) {
   if (qi < d.n_q && a.sp_active[qi]) {
     const int u = d.q_verts[qi];
     d.diag[u] = d.diagL[u] + (T)d.k_spring;
+    if (d.tm_springs) atomicAdd(&d.tm_springs[d.robot_of_vert ? d.robot_of_vert[u] : 0], 1);
   }
 }
 

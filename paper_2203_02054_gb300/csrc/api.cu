@@ -207,6 +207,47 @@ struct AAState {
   double* partials = nullptr;
 };
 
+// Team PCG (team.cu): how the free rows are cut into parts, and the tables
+// built from that at upload.
+struct TeamHost {
+  bool fits = false;
+  bool cluster = false;  // one thread-block cluster (a single robot of few parts)
+  int r_per = 1;   // rows per thread
+  int rows = 96;   // rows per part at most (what the threads of a block hold)
+  int threads = 192, grid = 1;
+  std::vector<TeamPart> part;
+  std::vector<int> halo;
+  std::vector<unsigned short> lcol;
+  std::vector<float4> z;
+  std::vector<double> Ac;         // the robots' coarse matrices
+  std::vector<long long> ac_off;
+  std::vector<int> ac_dim;
+  int halo_max = 0, max_np = 0;
+  bool coarse = false;
+  bool constants = false;  // coarse basis of constants alone, without sigma
+  size_t smem = 0;
+  int ainv_off = 0, val_off = 0, lcol_off = 0;
+  // length of a robot's parts: as few parts as possible, equally long (a
+  // round takes as long as the longest), in whole warps
+  int part_rows(int robot_rows) const {
+    const int np = std::max(1, (robot_rows + rows - 1) / rows);
+    return ((robot_rows + np - 1) / np + 31) & ~31;
+  }
+};
+struct TeamDevice {
+  TeamPart* part = nullptr;
+  int* halo = nullptr;
+  unsigned short* lcol = nullptr;
+  float4* z = nullptr;
+  float* ainv = nullptr;
+  size_t ainv_level = 0;
+  int* springs = nullptr;
+  unsigned long long *u = nullptr, *slot = nullptr;
+  unsigned* count = nullptr;
+  size_t zero_bytes = 0;
+  R4<double>*b = nullptr, *r = nullptr;
+};
+
 struct casim_sim {
   casim_params params{};
   std::vector<double> knots;
@@ -238,7 +279,7 @@ struct casim_sim {
   void *r = nullptr, *u = nullptr, *p = nullptr, *s = nullptr, *w = nullptr, *dx = nullptr, *spring_c = nullptr;
   void* pos_out = nullptr;
   void* X0 = nullptr;  // positions restored by casim_reset
-  void* xstep = nullptr;  // the last outer iteration's step per free row (MIXED warm start of the dataflow and batch PCG)
+  void* xstep = nullptr;  // the last outer iteration's step per free row (MIXED warm start of the team and batch PCG)
   int4 *tet = nullptr, *faces = nullptr;
   int *inc_ptr = nullptr, *inc = nullptr, *sl_ptr = nullptr, *sl_col = nullptr;
   int *q_verts_d = nullptr, *qf_ptr = nullptr, *qf = nullptr;
@@ -257,16 +298,9 @@ struct casim_sim {
   int cap_items = 0, n_slices = 0, pcg_grid = 1, n_e_local = 0, n_e_spring = 0;
   bool pcg_rr = false;  // register-resident PCG (one row per thread)
   bool pcg_cl = false;  // cluster PCG (one cluster per robot, work queue)
-  int pcg_variant = 1;  // whole-grid kernel: 1 streaming, 2 register-resident, 5 dataflow
-  unsigned long long *df_u = nullptr, *df_p = nullptr;  // dataflow PCG: epoch-tagged words
-  int *halo_ptr = nullptr, *halo_rows = nullptr, *sl_lcol = nullptr;  // dataflow PCG: block halos
-  int *halo_own = nullptr, *halo_self = nullptr;
-  std::vector<int> halo_ptr_h, halo_rows_h, sl_lcol_h, halo_own_h, halo_self_h;
-  int halo_max = 0;
-  int df_rows = 384;  // rows per block of the dataflow PCG
-  std::vector<float> cg_ainv_h;  // dataflow PCG coarse correction: A_c^-1, row-major
-  int n_agg = 0;
-  float* cg_ainv = nullptr;
+  int pcg_variant = 1;  // whole-grid kernel: 1 streaming, 2 register-resident, 5 team
+  TeamHost team;  // team PCG: plan and host-side tables of the upload
+  TeamDevice tm;
   bool pcg_seg = false; // segmented streaming PCG (batches: blocks per robot)
   int seg_blocks = 0;
   std::vector<int> seg_h;  // 5 x seg_blocks: lo, hi, rb0, rb1, robot
@@ -426,17 +460,32 @@ Dev<T> make_dev(casim_sim* sim) {
   d.w = (R4<T>*)sim->w;
   d.dx = (R4<T>*)sim->dx;
   d.partials = sim->partials;
-  d.df_u = sim->df_u;
-  d.df_p = sim->df_p;
-  d.halo_ptr = sim->halo_ptr;
-  d.halo_rows = sim->halo_rows;
-  d.halo_own = sim->halo_own;
-  d.halo_self = sim->halo_self;
-  d.sl_lcol = sim->sl_lcol;
-  d.halo_max = sim->halo_max;
-  d.df_rows = sim->df_rows;
-  d.cg_ainv = sim->cg_ainv;
-  d.n_agg = sim->n_agg;
+  d.tm_part = sim->tm.part;
+  d.tm_parts = (int)sim->team.part.size();
+  d.tm_grid = sim->team.grid;
+  d.tm_threads = sim->team.threads;
+  d.tm_r_per = sim->team.r_per;
+  d.tm_row_threads = sim->team.rows / sim->team.r_per;
+  d.tm_smem = (int)sim->team.smem;
+  d.tm_ainv_off = sim->team.ainv_off;
+  d.tm_val_off = sim->team.val_off;
+  d.tm_lcol_off = sim->team.lcol_off;
+  d.tm_cluster = sim->team.cluster;
+  d.tm_coarse = sim->team.coarse ? 1 : 0;
+  d.tm_levels = sim->team.constants ? 1 : TEAM_LEVELS;
+  d.tm_halo_max = sim->team.halo_max;
+  d.tm_halo = sim->tm.halo;
+  d.tm_lcol = sim->tm.lcol;
+  d.tm_z = sim->tm.z;
+  d.tm_ainv = sim->tm.ainv;
+  d.tm_ainv_level = sim->tm.ainv_level;
+  d.tm_springs = sim->tm.springs;
+  d.tm_u = sim->tm.u;
+  d.tm_slot = sim->tm.slot;
+  d.tm_count = sim->tm.count;
+  d.tm_zero_bytes = sim->tm.zero_bytes;
+  d.tm_b = sim->tm.b;
+  d.tm_r = sim->tm.r;
   d.q_verts = sim->q_verts_d;
   d.qf_ptr = sim->qf_ptr;
   d.qf = sim->qf;
@@ -501,7 +550,7 @@ Dev<T> make_dev(casim_sim* sim) {
   d.rhs_threads = sim->params.rhs_block ? sim->params.rhs_block : RHS_THREADS;
   d.narrow_threads = sim->params.narrow_block ? sim->params.narrow_block : 256;
   d.n_e_local = local_blocks(sim->n_t, d.local_threads);
-  d.n_e_spring = rhs_blocks(sim->n_free, d.rhs_threads);
+  d.n_e_spring = sim->pcg_variant == 5 ? d.tm_parts : rhs_blocks(sim->n_free, d.rhs_threads);
   return d;
 }
 
@@ -560,7 +609,9 @@ cudaError_t upload_spheres(casim_sim* sim) {
 // reads only the positions, which no collision kernel writes, and writes
 // only the projections P and its energy partials, which the collision
 // kernels do not read; the iteration's record takes both sides' terms by
-// integer atomics.  The global solve waits for both branches.
+// integer atomics.  The part of the team PCG's right-hand side that does not
+// depend on the springs and the clearing of its words follow it on that
+// branch.  The global solve waits for both branches.
 // NVTX range for profilers (a no-op unless a tool is attached); in graph
 // replay the ranges mark the capture, in eager mode every iteration.
 struct NvtxRange {
@@ -572,17 +623,27 @@ template <typename T>
 cudaError_t enqueue_iteration(casim_sim* sim, cudaStream_t st, cudaEvent_t* ev, cudaStream_t side = nullptr) {
   NvtxRange outer("casim iteration");
   const Dev<T> d = make_dev<T>(sim);
+  // the team PCG: its right-hand side is gathered beside the spring update,
+  // and with one robot it writes the iteration's record itself
+  const bool team = sim->pcg_variant == 5;
   if (ev) cudaEventRecord(ev[0], st);
   if (d.collision >= 1 && d.n_q > 0) {
     NvtxRange r("collision check");
     launch_collision<T>(d, sim->cs, st);
   }
   if (ev) cudaEventRecord(ev[1], st);
+  Dev<T> dp = d;
+  dp.rhs_in_pcg = team ? 1 : 0;
+  dp.xstep = (team || sim->pcg_seg) ? (R4<T>*)sim->xstep : nullptr;
   if (side) {
     cudaEventRecord(sim->ev_fork, st);
     cudaStreamWaitEvent(side, sim->ev_fork, 0);
-    NvtxRange r("local step");
-    launch_local<T>(d, side);
+    if (team) launch_team_clear<T>(dp, side);
+    {
+      NvtxRange r("local step");
+      launch_local<T>(d, side);
+    }
+    if (team) launch_team_rhs<T>(dp, side);
     cudaEventRecord(sim->ev_join, side);
   }
   if (d.collision >= 1 && d.n_q > 0) {
@@ -597,27 +658,91 @@ cudaError_t enqueue_iteration(casim_sim* sim, cudaStream_t st, cudaEvent_t* ev, 
     launch_local<T>(d, st);
   }
   if (ev) cudaEventRecord(ev[3], st);
-  // the dataflow PCG forms the right-hand side, the diagonal and the
-  // iteration's record itself (one launch instead of three)
-  const bool fused = !sim->pcg_seg && !sim->pcg_cl && sim->pcg_variant == 5;
-  if (!fused) {
+  if (!team) {
     NvtxRange r("rhs gather");
     launch_rhs<T>(d, st);
+  } else if (!side) {
+    NvtxRange r("rhs gather");
+    launch_team_clear<T>(dp, st);
+    launch_team_rhs<T>(dp, st);
   }
   if (ev) cudaEventRecord(ev[4], st);
   NvtxRange rp("global solve");
-  // reset the grid-barrier words (abort, count, generation) before the PCG
+  // reset the abort and grid-barrier words before the PCG
   cudaMemsetAsync(reinterpret_cast<char*>(sim->ctrl) + offsetof(Ctrl, abort), 0, 3 * sizeof(int), st);
-  Dev<T> dp = d;
-  dp.rhs_in_pcg = fused ? 1 : 0;
-  dp.xstep = (fused || sim->pcg_seg) ? (R4<T>*)sim->xstep : nullptr;
-  cudaError_t e = sim->pcg_seg  ? launch_pcg_seg<T>(dp, sim->seg_blocks, st)
-                  : sim->pcg_cl ? launch_pcg_cluster<T>(d, sim->pcg_clusters, st)
-                                : launch_pcg<T>(dp, sim->pcg_grid, sim->pcg_variant, st);
+  cudaError_t e = team            ? launch_pcg_team<T>(dp, st)
+                  : sim->pcg_seg  ? launch_pcg_seg<T>(dp, sim->seg_blocks, st)
+                  : sim->pcg_cl   ? launch_pcg_cluster<T>(d, sim->pcg_clusters, st)
+                                  : launch_pcg<T>(dp, sim->pcg_grid, sim->pcg_variant, st);
   if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[5], st);
-  if (!fused) launch_finalize<T>(d, st);
+  if (!team || d.n_robots > 1) launch_finalize<T>(d, st);
   return cudaGetLastError();
+}
+
+// The team PCG's tables, and the inverses of its coarse matrices (on the
+// device; a matrix that is not positive definite leaves Jacobi alone).
+int upload_team(casim_sim* sim) {
+  TeamHost& h = sim->team;
+  TeamDevice& g = sim->tm;
+  cudaStream_t st = sim->stream;
+  auto up = [&](void* dst, const void* src, size_t bytes) {
+    return bytes ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st) : cudaSuccess;
+  };
+  CK(cudaMemsetAsync(g.springs, 0, sizeof(int) * sim->n_robots, st));
+  CK(up(g.part, h.part.data(), sizeof(TeamPart) * h.part.size()));
+  CK(up(g.halo, h.halo.data(), sizeof(int) * h.halo.size()));
+  CK(up(g.lcol, h.lcol.data(), sizeof(unsigned short) * h.lcol.size()));
+  if (h.coarse) {
+    const int nm = (int)h.ac_dim.size();
+    const int mx = *std::max_element(h.ac_dim.begin(), h.ac_dim.end());
+    CK(up(g.z, h.z.data(), sizeof(float4) * h.z.size()));
+    // one matrix per level and robot: A_c + sigma I; scratch of the inversion:
+    // matrices, panels, pivots, offsets, dimensions, flags
+    const int n = TEAM_LEVELS * nm;
+    const size_t nl = h.Ac.size(), nA = TEAM_LEVELS * nl, nC = (size_t)n * mx * 32, nD = (size_t)n * 32 * 32;
+    char* tmp = nullptr;
+    const size_t bytes = sizeof(double) * (nA + nC + nD) + sizeof(long long) * n + 2 * sizeof(int) * (size_t)n;
+    CK(cudaMalloc(&tmp, bytes));
+    double* A = reinterpret_cast<double*>(tmp);
+    double *C = A + nA, *D = C + nC;
+    long long* off = reinterpret_cast<long long*>(D + nD);
+    int *dim = reinterpret_cast<int*>(off + n), *bad = dim + n;
+    std::vector<int> bad_h(n, 0), dim_h;
+    std::vector<long long> off_h;
+    std::vector<double> shift(TEAM_LEVELS, 0.0);
+    for (int l = 0; l < TEAM_LEVELS; ++l) {
+      if (l) shift[l] = sim->params.k_spring * TEAM_SIGMA_1 * std::pow(4.0, l - 1);
+      for (int r = 0; r < nm; ++r) {
+        off_h.push_back(h.ac_off[r] + (long long)(l * nl));
+        dim_h.push_back(h.ac_dim[r]);
+      }
+    }
+    cudaError_t e = up(A, h.Ac.data(), sizeof(double) * nl);
+    for (int l = 1; l < TEAM_LEVELS && e == cudaSuccess; ++l)
+      e = cudaMemcpyAsync(A + l * nl, A, sizeof(double) * nl, cudaMemcpyDeviceToDevice, st);
+    if (e == cudaSuccess) e = up(off, off_h.data(), sizeof(long long) * n);
+    if (e == cudaSuccess) e = up(dim, dim_h.data(), sizeof(int) * n);
+    if (e == cudaSuccess) e = cudaMemsetAsync(bad, 0, sizeof(int) * n, st);
+    if (e == cudaSuccess) {
+      for (int l = 1; l < TEAM_LEVELS; ++l) launch_shift(A, off + l * nm, dim + l * nm, nm, shift[l], st);
+      launch_invert(A, off, dim, n, mx, C, D, g.ainv, bad, st);
+      e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(bad_h.data(), bad, sizeof(int) * n, cudaMemcpyDeviceToHost, st);
+    const cudaError_t e2 = cudaStreamSynchronize(st);
+    cudaFree(tmp);
+    CK(e);
+    CK(e2);
+    for (int b : bad_h)
+      if (b) h.coarse = false;
+  }
+  CK(cudaStreamSynchronize(st));
+  h.halo = {};
+  h.lcol = {};
+  h.z = {};
+  h.Ac = {};
+  return CASIM_OK;
 }
 
 template <typename T>
@@ -658,21 +783,34 @@ int upload_typed(casim_sim* sim, const std::vector<double>& rest_int, const std:
   sim->s = sim->dalloc<R4<T>>(n_free);
   sim->w = sim->dalloc<R4<T>>(n_free);
   sim->dx = sim->dalloc<R4<T>>(n_free);
-  // the step that the next solve starts from (MIXED; dataflow and batch PCG)
+  // the step that the next solve starts from (MIXED; team and batch PCG)
   sim->xstep = std::is_same<T, float>::value && (sim->pcg_variant == 5 || sim->pcg_seg)
                    ? sim->dalloc<R4<T>>(std::max(n_free, 1))
                    : nullptr;
   sim->spring_c = sim->dalloc<R4<double>>(n_free);
   sim->partials = sim->dalloc<double>(2 * 4 * (size_t)std::max(sim->pcg_grid, 1));
+  sim->tm = TeamDevice{};
   if (sim->pcg_variant == 5) {
-    sim->df_u = sim->dalloc<unsigned long long>(4 * (size_t)std::max(n_free, 1));
-    sim->df_p = sim->dalloc<unsigned long long>((size_t)PCG_DF_REPLICAS * 2 * 16 * ((size_t)sim->pcg_grid + 1));
-    if (sim->n_agg > 0) sim->cg_ainv = sim->dalloc<float>((size_t)sim->n_agg * sim->n_agg);
-    sim->halo_ptr = sim->dalloc<int>(sim->halo_ptr_h.size());
-    sim->halo_rows = sim->dalloc<int>(std::max<size_t>(sim->halo_rows_h.size(), 1));
-    sim->sl_lcol = sim->dalloc<int>(std::max<size_t>(sim->sl_lcol_h.size(), 1));
-    sim->halo_own = sim->dalloc<int>(std::max<size_t>(sim->halo_own_h.size(), 1));
-    sim->halo_self = sim->dalloc<int>(std::max<size_t>(sim->halo_self_h.size(), 1));
+    const TeamHost& h = sim->team;
+    TeamDevice& g = sim->tm;
+    size_t slot_off = 0, count_off = 0;
+    const size_t words = team_words(!std::is_same<T, float>::value, n_free, (int)h.part.size(), sim->n_robots,
+                                    slot_off, count_off);
+    g.part = sim->dalloc<TeamPart>(h.part.size());
+    g.halo = sim->dalloc<int>(h.halo.size());
+    g.lcol = sim->dalloc<unsigned short>(h.lcol.size());
+    g.u = sim->dalloc<unsigned long long>(words);
+    g.slot = g.u + slot_off;
+    g.count = reinterpret_cast<unsigned*>(g.u + count_off);
+    g.zero_bytes = sizeof(unsigned long long) * words;
+    g.b = sim->dalloc<R4<double>>(n_free);
+    g.r = sim->dalloc<R4<double>>(n_free);
+    if (h.coarse) {
+      g.z = sim->dalloc<float4>(n_free);
+      g.ainv = sim->dalloc<float>(TEAM_LEVELS * h.Ac.size());
+      g.ainv_level = h.Ac.size();
+    }
+    g.springs = sim->dalloc<int>(sim->n_robots);
   }
   sim->q_verts_d = sim->dalloc<int>(n_q);
   sim->qf_ptr = sim->dalloc<int>(n_q + 1);
@@ -744,13 +882,16 @@ int upload_typed(casim_sim* sim, const std::vector<double>& rest_int, const std:
   sim->hist = sim->dalloc<IterRec>(sim->hist_cap);
   // energy partials: room for the smallest allowed block sizes
   sim->n_e_local = local_blocks(n_t, 64);
-  sim->n_e_spring = rhs_blocks(n_free, 128);
+  sim->n_e_spring = std::max(rhs_blocks(n_free, 128), (int)sim->team.part.size());
   sim->e_partials = sim->dalloc<double>(sim->n_e_local + sim->n_e_spring + 1);
   alloc_bvh(sim->bvh_t_h, n_t, 4, sim->tet, sim->bt);
   alloc_bvh(sim->bvh_f_h, n_f, 3, sim->faces, sim->bf);
   for (void* q : sim->allocs)
     if (!q) return sim->fail(CASIM_E_CUDA, "cudaMalloc failed");
-  if (!sim->X || !sim->items || !sim->P || !sim->e_partials || !sim->hist)
+  const bool team_lost = sim->pcg_variant == 5 &&
+                         (!sim->tm.part || !sim->tm.halo || !sim->tm.lcol || !sim->tm.u || !sim->tm.b || !sim->tm.r || !sim->tm.springs ||
+                          (sim->team.coarse && (!sim->tm.z || !sim->tm.ainv)));
+  if (!sim->X || !sim->items || !sim->P || !sim->e_partials || !sim->hist || team_lost)
     return sim->fail(CASIM_E_CUDA, "device allocation failed");
 
   std::vector<R4<T>> Xh(n_v);
@@ -797,23 +938,8 @@ int upload_typed(casim_sim* sim, const std::vector<double>& rest_int, const std:
     CK(cudaMemcpyAsync(sim->sl_val, slv.data(), sizeof(T) * slv.size(), cudaMemcpyHostToDevice, st));
   }
   if (sim->pcg_variant == 5) {
-    CK(cudaMemcpyAsync(sim->halo_ptr, sim->halo_ptr_h.data(), sizeof(int) * sim->halo_ptr_h.size(),
-                       cudaMemcpyHostToDevice, st));
-    if (!sim->halo_rows_h.empty())
-      CK(cudaMemcpyAsync(sim->halo_rows, sim->halo_rows_h.data(), sizeof(int) * sim->halo_rows_h.size(),
-                         cudaMemcpyHostToDevice, st));
-    if (!sim->sl_lcol_h.empty())
-      CK(cudaMemcpyAsync(sim->sl_lcol, sim->sl_lcol_h.data(), sizeof(int) * sim->sl_lcol_h.size(),
-                         cudaMemcpyHostToDevice, st));
-    if (!sim->halo_own_h.empty())
-      CK(cudaMemcpyAsync(sim->halo_own, sim->halo_own_h.data(), sizeof(int) * sim->halo_own_h.size(),
-                         cudaMemcpyHostToDevice, st));
-    if (!sim->halo_self_h.empty())
-      CK(cudaMemcpyAsync(sim->halo_self, sim->halo_self_h.data(), sizeof(int) * sim->halo_self_h.size(),
-                         cudaMemcpyHostToDevice, st));
-    if (sim->n_agg > 0)
-      CK(cudaMemcpyAsync(sim->cg_ainv, sim->cg_ainv_h.data(), sizeof(float) * sim->cg_ainv_h.size(),
-                         cudaMemcpyHostToDevice, st));
+    const int rc = upload_team(sim);
+    if (rc) return rc;
   }
   if (n_q) {
     CK(cudaMemcpyAsync(sim->q_verts_d, sim->q_verts.data(), sizeof(int) * n_q, cudaMemcpyHostToDevice, st));
@@ -1265,6 +1391,8 @@ int backward_typed(casim_sim* sim, const double* dL_dX, double* dL_dalpha) {
     const int m = std::min(A.every, A.n_iters - first);
     CK((adj_copy_state<T>(sim, (R4<T>*)A.ckX + c * nv, A.ck_act + c * nq, A.ck_kind + c * nq, A.ck_face + c * nq,
                           A.ck_bary + c * 2 * nq, A.ck_tgt + c * 3 * nq, false)));
+    // (outer iterations count their springs from zero)
+    if (sim->tm.springs) CK(cudaMemsetAsync(sim->tm.springs, 0, sizeof(int) * sim->n_robots, st));
     // recompute the segment, keeping X_i and the spring decisions of each iteration
     for (int j = 0; j < m; ++j) {
       CK(cudaMemcpyAsync((R4<T>*)A.segX + j * nv, sim->X, sizeof(R4<T>) * nv, cudaMemcpyDeviceToDevice, st));
@@ -1311,12 +1439,16 @@ int backward_typed(casim_sim* sim, const double* dL_dX, double* dL_dalpha) {
       if (sim->params.collision == 0 || sim->n_q == 0) {
         CK(cudaMemsetAsync(A.seg_act + j * nq, 0, sizeof(int) * nq, st));
       }
+      if (sim->tm.springs) CK(cudaMemsetAsync(sim->tm.springs, 0, sizeof(int) * sim->n_robots, st));
       launch_adjoint_diag<T>(d, a, st);
       CK(cudaMemsetAsync(A.mu, 0, sizeof(R4<T>) * std::max(nf, 1), st));
       CK(cudaMemsetAsync(reinterpret_cast<char*>(sim->ctrl) + offsetof(Ctrl, abort), 0, 3 * sizeof(int), st));
-      cudaError_t e = sim->pcg_seg  ? launch_pcg_seg<T>(dpcg, sim->seg_blocks, st)
-                      : sim->pcg_cl ? launch_pcg_cluster<T>(dpcg, sim->pcg_clusters, st)
-                                    : launch_pcg<T>(dpcg, sim->pcg_grid, sim->pcg_variant, st);
+      const bool team = sim->pcg_variant == 5;
+      if (team) CK(launch_team_clear<T>(dpcg, st));
+      cudaError_t e = team            ? launch_pcg_team<T>(dpcg, st)
+                      : sim->pcg_seg  ? launch_pcg_seg<T>(dpcg, sim->seg_blocks, st)
+                      : sim->pcg_cl   ? launch_pcg_cluster<T>(dpcg, sim->pcg_clusters, st)
+                                      : launch_pcg<T>(dpcg, sim->pcg_grid, sim->pcg_variant, st);
       if (e != cudaSuccess) return sim->fail(CASIM_E_CUDA, std::string("adjoint solve: ") + cudaGetErrorString(e));
       launch_adjoint_step<T>(d, a, st);
       CK(cudaGetLastError());
@@ -1324,6 +1456,7 @@ int backward_typed(casim_sim* sim, const double* dL_dX, double* dL_dalpha) {
   }
   std::vector<double> ab(std::max(ng, 1));
   if (ng) CK(cudaMemcpyAsync(ab.data(), A.abar, sizeof(double) * ng, cudaMemcpyDeviceToHost, st));
+  if (sim->tm.springs) CK(cudaMemsetAsync(sim->tm.springs, 0, sizeof(int) * sim->n_robots, st));
   // restore the final forward state and the counters
   CK((adj_copy_state<T>(sim, A.finX, A.fin_act, A.fin_kind, A.fin_face, A.fin_bary, A.fin_tgt, false)));
   int st_bits = 0;
@@ -1336,6 +1469,220 @@ int backward_typed(casim_sim* sim, const double* dL_dX, double* dL_dalpha) {
   for (int gi = 0; gi < ng; ++gi) dL_dalpha[gi] = ab[gi];
   if (st_bits & (ST_TIMEOUT | ST_NONFINITE)) return sim->fail(CASIM_E_NONFINITE, "adjoint pass: device status");
   return CASIM_OK;
+}
+
+int device_sms() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
+// Cuts the robots' free rows (rows[r] of robot r) into parts of equal length
+// for the team PCG: the shortest parts with which every block of the grid (one
+// per SM) has at most one; when even the longest leave more than that, the
+// blocks work through several robots' parts in turn.  Short parts make the
+// coarse space finer and an SM's share of the work smaller, long ones the rounds
+// cheaper: a 10,959-row finger took 696 CG iterations over a run and 97 us per
+// solve with parts of 96 rows (115 blocks), 685 and 96 us with 128, 775 and 109
+// us with 192, 862 and 120 us with 288 (39 blocks).  FP64 may go down to 32 rows
+// (a 500-row beam: 33 iterations and 314 us per solve; 367 us with 64, 400 us
+// with 96), FP32 stops at 96.
+void plan_team(const casim_params& p, const std::vector<int>& rows, TeamHost& h) {
+  h = TeamHost{};
+  const bool fp64 = p.precision == CASIM_FP64;
+  const int sms = std::min(device_sms(), TEAM_MAX_PARTS);
+  if (sms < 1) return;
+  const int biggest = *std::max_element(rows.begin(), rows.end());
+  if (biggest < 1) return;
+  auto parts = [&](int len) {
+    long long n = 0;
+    for (int r : rows) n += (r + len - 1) / len;
+    return n;
+  };
+  auto take = [&](int r_per, int len) {
+    h.r_per = r_per;
+    h.rows = len;
+    h.fits = (biggest + len - 1) / len <= sms;
+    // at least a warp for the scalars and a thread per slot beside it
+    h.threads = std::max(len / r_per * (fp64 ? 3 : 1), 192);
+    return h.fits;
+  };
+  if (fp64) {
+    for (int r = 1; r <= 3; ++r)
+      for (int rt = r == 1 ? 32 : 96; 3 * rt <= TEAM_NT_F64; rt += 32)
+        if (parts(r * rt) <= sms) {
+          take(r, r * rt);
+          return;
+        }
+    take(3, TEAM_NT_F64);
+    return;
+  }
+  if (p.pcg_block) {
+    take(1, p.pcg_block);
+    return;
+  }
+  for (int len = 96; len <= TEAM_NT_1; len += 32)
+    if (parts(len) <= sms) {
+      take(1, len);
+      return;
+    }
+  for (int nt = 192; nt <= TEAM_NT_3; nt += 32)
+    if (parts(3 * nt) <= sms) {
+      take(3, 3 * nt);
+      return;
+    }
+  take(3, 3 * TEAM_NT_3);
+}
+
+// The parts, their halos (own rows first, then the other parts' rows that
+// their rows read, ascending), every sliced-ELL entry's index in its part's
+// halo, the coarse basis and the Galerkin matrices.
+void build_team(casim_sim* sim, const std::vector<double>& rest_int,
+                const std::vector<std::vector<std::pair<int, double>>>& rows_ff, const std::vector<double>& diagL,
+                const std::vector<int>& sl_ptr, const std::vector<int>& sl_col, int max_width) {
+  TeamHost& h = sim->team;
+  const bool fp64 = sim->params.precision == CASIM_FP64;
+  const int n_free = sim->n_free;
+  std::vector<int> part_of(n_free);
+  for (int r = 0; r < sim->n_robots; ++r) {
+    const int a = sim->robot_row_h[r], b = sim->robot_row_h[r + 1];
+    const int len = h.part_rows(b - a), p0 = (int)h.part.size(), np = (b - a + len - 1) / len;
+    h.max_np = std::max(h.max_np, np);
+    for (int k = 0; k < np; ++k) {
+      TeamPart t{};
+      t.robot = r;
+      t.p0 = p0;
+      t.np = np;
+      t.row0 = a + k * len;
+      t.nrow = std::min(len, b - t.row0);
+      for (int i = 0; i < t.nrow; ++i) part_of[t.row0 + i] = (int)h.part.size();
+      h.part.push_back(t);
+    }
+  }
+  h.grid = std::max(1, std::min((int)h.part.size(), device_sms()));
+  h.lcol.assign(std::max<size_t>(sl_col.size(), 1), 0);
+  std::vector<int> seen(n_free, -1), local(n_free, 0), other;
+  for (int p = 0; p < (int)h.part.size(); ++p) {
+    TeamPart& t = h.part[p];
+    other.clear();
+    auto each = [&](auto fn) {
+      for (int i = t.row0; i < t.row0 + t.nrow; ++i)
+        for (int k = sl_ptr[i >> 5] + (i & 31); k < sl_ptr[(i >> 5) + 1]; k += 32) fn(k, sl_col[k]);
+    };
+    each([&](int, int c) {
+      if ((c < t.row0 || c >= t.row0 + t.nrow) && seen[c] != p) {
+        seen[c] = p;
+        other.push_back(c);
+      }
+    });
+    std::sort(other.begin(), other.end());
+    for (size_t j = 0; j < other.size(); ++j) local[other[j]] = t.nrow + (int)j;
+    t.halo0 = (int)h.halo.size();
+    t.n_other = (int)other.size();
+    h.halo.insert(h.halo.end(), other.begin(), other.end());
+    h.halo_max = std::max(h.halo_max, t.nrow + t.n_other);
+    if (t.nrow + t.n_other > 65535 || (fp64 ? 3 : 1) * t.n_other > 64 * h.threads) {
+      h.fits = false;
+      return;
+    }
+    each([&](int k, int c) {
+      h.lcol[k] = (unsigned short)(c >= t.row0 && c < t.row0 + t.nrow ? c - t.row0 : local[c]);
+    });
+  }
+  if (h.halo.empty()) h.halo.push_back(0);
+  h.coarse = sim->params.pcg_precond == 0;
+  // Small single robots in MIXED keep the constants alone over 96 rows, without
+  // sigma: their runs are decided by single contacts (one decision that falls
+  // the other way moves a 570-vertex finger by 5e-5 of its size), so a solve
+  // that leaves another error of the same size within the tolerance changes
+  // where a twelfth of the runs go (7 of 80 over ten iterations); with this
+  // basis they follow the trajectories they always did.
+  h.constants = !fp64 && sim->n_robots == 1 && n_free <= TEAM_CONSTANTS_MAX;
+  if (h.coarse) {
+    // basis of every part: 1 and the rest coordinates, orthonormalised in that
+    // order; a function that depends on the earlier ones (a part with fewer
+    // than four rows, or a flat one) becomes zero, its diagonal entry one
+    h.z.assign(std::max(n_free, 1), make_float4(0.0f, 0.0f, 0.0f, 0.0f));
+    std::vector<double> q;
+    std::vector<char> dead(4 * h.part.size(), 0);
+    for (size_t p = 0; p < h.part.size(); ++p) {
+      const int r0 = h.part[p].row0, m = h.part[p].nrow;
+      q.assign(4 * (size_t)m, 0.0);
+      for (int f = 0; f < 4; ++f) {
+        double* v = q.data() + (size_t)f * m;
+        double size = 0.0, left = 0.0;
+        for (int i = 0; i < m; ++i) {
+          v[i] = f == 0 ? 1.0 : rest_int[3 * (size_t)(r0 + i) + f - 1] - rest_int[3 * (size_t)r0 + f - 1];
+          size += v[i] * v[i];
+        }
+        for (int pass = 0; pass < 2; ++pass)
+          for (int g = 0; g < f; ++g) {
+            const double* w = q.data() + (size_t)g * m;
+            double c = 0.0;
+            for (int i = 0; i < m; ++i) c += v[i] * w[i];
+            for (int i = 0; i < m; ++i) v[i] -= c * w[i];
+          }
+        for (int i = 0; i < m; ++i) left += v[i] * v[i];
+        const bool ok = left > 1e-12 * size && left > 0.0 && !(h.constants && f > 0);
+        const double s = ok ? 1.0 / std::sqrt(left) : 0.0;
+        for (int i = 0; i < m; ++i) {
+          v[i] *= s;
+          (&h.z[r0 + i].x)[f] = (float)v[i];
+        }
+        if (!ok) dead[4 * p + f] = 1;
+      }
+    }
+    // A_c = Z^T L Z per robot: for every row the sums of its entries times the
+    // basis of each part they reach, then the outer products
+    std::vector<long long> off(1, 0);
+    for (int r = 0; r < sim->n_robots; ++r) {
+      const int rows = sim->robot_row_h[r + 1] - sim->robot_row_h[r], len = h.part_rows(rows);
+      const long long nd = 4LL * ((rows + len - 1) / len);
+      h.ac_dim.push_back((int)nd);
+      h.ac_off.push_back(off.back());
+      off.push_back(off.back() + nd * nd);
+    }
+    h.Ac.assign(std::max<size_t>((size_t)off.back(), 1), 0.0);
+    struct Reach {
+      int part;
+      double v[4];
+    };
+    std::vector<Reach> reach;
+    for (size_t p = 0; p < h.part.size(); ++p) {
+      TeamPart& t = h.part[p];
+      const long long nd = 4LL * t.np;
+      double* Ac = h.Ac.data() + h.ac_off[t.robot];
+      t.ainv = h.ac_off[t.robot] + 4LL * ((long long)p - t.p0) * nd;
+      const int a = (int)p - t.p0;
+      for (int i = t.row0; i < t.row0 + t.nrow; ++i) {
+        reach.clear();
+        auto add = [&](int row, double val) {
+          const int b = part_of[row] - t.p0;
+          size_t k = 0;
+          while (k < reach.size() && reach[k].part != b) ++k;
+          if (k == reach.size()) reach.push_back(Reach{b, {0, 0, 0, 0}});
+          for (int f = 0; f < 4; ++f) reach[k].v[f] += val * (double)(&h.z[row].x)[f];
+        };
+        add(i, diagL[i]);
+        for (const auto& e : rows_ff[i]) add(e.first, e.second);
+        for (const Reach& k : reach)
+          for (int f = 0; f < 4; ++f)
+            for (int g = 0; g < 4; ++g)
+              Ac[(4LL * a + f) * nd + 4LL * k.part + g] += (double)(&h.z[i].x)[f] * k.v[g];
+      }
+      for (int f = 0; f < 4; ++f)
+        if (dead[4 * p + f]) Ac[(4LL * a + f) * (nd + 1)] = 1.0;
+    }
+  }
+  h.smem = team_smem(fp64, h.rows, h.r_per, h.halo_max, h.max_np, h.coarse, max_width, h.ainv_off,
+                     h.val_off, h.lcol_off);
+  // a small team in one cluster (not under the test-only fault injection: the
+  // hardware barrier has no wait to run out)
+  h.cluster = sim->n_robots == 1 && h.r_per == 1 && (int)h.part.size() <= TEAM_CLUSTER &&
+              !(sim->params.debug_flags & CASIM_DEBUG_BARRIER_NEVER_COMPLETES) && h.smem <= TEAM_SMEM_MAX &&
+              team_prepare(fp64, h.r_per, true, h.grid, h.threads, h.smem);
+  h.fits = h.cluster || (h.smem <= TEAM_SMEM_MAX && team_prepare(fp64, h.r_per, false, h.grid, h.threads, h.smem));
 }
 
 }  // namespace
@@ -1449,22 +1796,18 @@ static int upload_robots(casim_sim* sim, int32_t n_verts, const double* rest_xyz
   sim->user_of_int.assign(n_v, -1);
   int nf = 0;
   {
-    // rows per block of the dataflow PCG (single robot, MIXED): 288 (9 warps,
-    // more blocks, fewer rows each) when the system fits 152 such blocks,
-    // else 384; the bisection leaves are its aggregates (a third of a block)
-    int n_free_all = 0;
-    for (int v = 0; v < n_v; ++v) n_free_all += !fixed[v];
-    const int pb = sim->params.pcg_block;
-    sim->df_rows = (pb == PCG_DF_THREADS || (pb == 0 && n_free_all > pcg_df_max_rows(PCG_DF_ROWS_SMALL)))
-                       ? PCG_DF_THREADS
-                       : PCG_DF_ROWS_SMALL;
-    const int leaf = n_robots == 1 ? sim->df_rows / 3 : 128;
+    std::vector<int> rows(n_robots, 0);
+    for (int v = 0; v < n_v; ++v)
+      if (!fixed[v]) rows[std::max(0, robot_of_vert_user[v])]++;
+    plan_team(sim->params, rows, sim->team);
+    // the bisection's leaves are the solver's parts
+    const bool parts = sim->params.pcg_kernel != 4 && sim->team.fits;
     std::vector<std::vector<int>> per_robot(n_robots);
     for (int v = 0; v < n_v; ++v)
       if (!fixed[v]) per_robot[std::max(0, robot_of_vert_user[v])].push_back(v);
     for (int r = 0; r < n_robots; ++r) {
       std::vector<int>& L = per_robot[r];
-      rcb_order(rest_xyz, L.data(), (int)L.size(), leaf);
+      rcb_order(rest_xyz, L.data(), (int)L.size(), parts ? sim->team.part_rows((int)L.size()) : 128);
       for (int v : L) sim->int_of_user[v] = nf++;
     }
   }
@@ -1661,78 +2004,14 @@ static int upload_robots(casim_sim* sim, int32_t n_verts, const double* rest_xyz
   const bool fp64 = sim->params.precision == CASIM_FP64;
   const int rr_rows = fp64 ? pcg_rr_max_rows<double>() : pcg_rr_max_rows<float>();
   const bool rr_fits = max_width <= PCG_RR_MAXW && n_free <= rr_rows;
-  // dataflow PCG (FP32 vectors only): one row per thread, one block per SM.
-  // Block b owns rows [b R, (b + 1) R), R = df_rows (whole slices); its
-  // halo is the list of distinct columns its rows read, its own rows first
-  // (each row writes its value there itself, from its registers), then the
-  // other blocks' rows it loads, each part ascending; every sliced-ELL entry
-  // also gets its column's index in that list.
-  const int R_df = sim->df_rows;
-  bool df_fits = !fp64 && max_width <= PCG_RR_MAXW && n_free <= pcg_df_max_rows(R_df);
-  sim->halo_ptr_h.clear();
-  sim->halo_rows_h.clear();
-  sim->sl_lcol_h.clear();
-  sim->halo_own_h.clear();
-  sim->halo_self_h.clear();
-  sim->halo_max = 0;
-  if (df_fits) {
-    const int spb = R_df / 32;
-    const int nbk = (n_free + R_df - 1) / R_df;
-    sim->halo_ptr_h.assign(nbk + 1, 0);
-    sim->halo_own_h.assign(nbk, 0);
-    sim->halo_self_h.assign(n_free, -1);
-    sim->sl_lcol_h.assign(sl_col.size(), 0);
-    std::vector<int> cols, own, other;
-    for (int b = 0; b < nbk; ++b) {
-      const int s0 = b * spb, s1 = std::min(sim->n_slices, s0 + spb);
-      const int r0 = b * R_df, r1 = r0 + R_df;
-      cols.clear();
-      for (int s = s0; s < s1; ++s)
-        for (int k = sl_ptr[s]; k < sl_ptr[s + 1]; ++k)
-          if (32 * s + (k - sl_ptr[s]) % 32 < n_free) cols.push_back(sl_col[k]);
-      std::sort(cols.begin(), cols.end());
-      cols.erase(std::unique(cols.begin(), cols.end()), cols.end());
-      own.clear();
-      other.clear();
-      for (int c : cols) (c >= r0 && c < r1 ? own : other).push_back(c);
-      const int n_own = (int)own.size();
-      for (int j = 0; j < n_own; ++j) sim->halo_self_h[own[j]] = j;
-      for (int s = s0; s < s1; ++s)
-        for (int k = sl_ptr[s]; k < sl_ptr[s + 1]; ++k)
-          if (32 * s + (k - sl_ptr[s]) % 32 < n_free) {
-            const int c = sl_col[k];
-            sim->sl_lcol_h[k] =
-                c >= r0 && c < r1 ? (int)(std::lower_bound(own.begin(), own.end(), c) - own.begin())
-                                  : n_own + (int)(std::lower_bound(other.begin(), other.end(), c) - other.begin());
-          }
-      sim->halo_rows_h.insert(sim->halo_rows_h.end(), own.begin(), own.end());
-      sim->halo_rows_h.insert(sim->halo_rows_h.end(), other.begin(), other.end());
-      sim->halo_ptr_h[b + 1] = (int)sim->halo_rows_h.size();
-      sim->halo_own_h[b] = n_own;
-      sim->halo_max = std::max(sim->halo_max, (int)cols.size());
-    }
-    if ((size_t)sim->halo_max * 16 > PCG_DF_HALO_MAX_BYTES) df_fits = false;
-  }
-  // two-level preconditioner of the dataflow kernel: Galerkin coarse matrix
-  // A_c = Z^T L Z of the free-row Laplacian over aggregates of consecutive
-  // rows (a = row / R), inverted here in FP64 (Cholesky)
-  sim->n_agg = 0;
-  sim->cg_ainv_h.clear();
-  if (df_fits && n_robots == 1 && sim->params.pcg_precond == 0) {
-    const int R = R_df / 3;
-    const int na = (n_free + R - 1) / R;
-    std::vector<double> Ac((size_t)na * na, 0.0);
-    for (int v = 0; v < n_free; ++v) {
-      const int a = v / R;
-      Ac[(size_t)a * na + a] += diagL[v];
-      for (const auto& e : rows_ff[v]) Ac[(size_t)a * na + e.first / R] += e.second;
-    }
-    if (cholesky_inverse(Ac, na)) {
-      sim->n_agg = na;
-      sim->cg_ainv_h.assign(Ac.begin(), Ac.end());
-    }
-  }
-  if (df_fits && !pcg_df_prepare(R_df, 16 * sim->halo_max + (int)sizeof(float) * 3 * sim->n_agg)) df_fits = false;
+  const int kern = sim->params.pcg_kernel;
+  // a forced team PCG keeps the limits of one FP32 row per thread
+  const bool team_ok = kern == 0 || (kern == 5 && !fp64 && n_free <= device_sms() * (sim->params.pcg_block == 288 ? 288 : 384));
+  TeamHost& team = sim->team;
+  if (team.fits && team_ok && max_width <= TEAM_MAX_WIDTH)
+    build_team(sim, rest_int, rows_ff, diagL, sl_ptr, sl_col, max_width);
+  else
+    team.fits = false;
   // cluster PCG: every robot's rows must fit the cluster's shared memory
   int max_robot_rows = 0;
   for (int r = 0; r < sim->n_robots; ++r)
@@ -1742,19 +2021,18 @@ static int upload_robots(casim_sim* sim, int32_t n_verts, const double* rest_xyz
   int max_clusters = 0;
   if (need <= cap) max_clusters = fp64 ? pcg_cluster_max_clusters<double>(cap) : pcg_cluster_max_clusters<float>(cap);
   const bool cl_fits = need <= cap && max_clusters > 0;
-  const int kern = sim->params.pcg_kernel;
-  if ((kern == 2 && !rr_fits) || (kern == 3 && !cl_fits) || (kern == 5 && !df_fits))
+  if ((kern == 2 && !rr_fits) || (kern == 3 && !cl_fits) || (kern == 5 && !team.fits))
     return sim->fail(CASIM_E_INVALID, "requested PCG kernel does not fit this mesh (" + std::to_string(n_free) +
                                           " rows, width " + std::to_string(max_width) + ")");
-  // auto: a single system runs fastest on the whole-grid register-resident
-  // kernel (latency bound); several robots share the GPU through the cluster
-  // kernel's work queue
+  // auto: the team PCG where it fits (vectors on chip, no grid barrier, one
+  // team per robot); systems beyond it run on the kernels that keep their
+  // vectors in memory, several robots with blocks assigned to robots
   const bool many = sim->n_robots > 1;
   // segmented streaming PCG: every robot needs at least one co-resident block
   const int seg_max = fp64 ? pcg_seg_max_blocks<double>() : pcg_seg_max_blocks<float>();
   const bool seg_fits = sim->n_robots <= seg_max && seg_max > 0;
   if (kern == 4 && !seg_fits) return sim->fail(CASIM_E_INVALID, "segmented PCG: more robots than co-resident blocks");
-  sim->pcg_seg = (kern == 4) || (kern == 0 && many && seg_fits);
+  sim->pcg_seg = (kern == 4) || (kern == 0 && !team.fits && many && seg_fits);
   sim->seg_h.clear();
   sim->seg_blocks = 0;
   if (sim->pcg_seg) {
@@ -1866,16 +2144,17 @@ static int upload_robots(casim_sim* sim, int32_t n_verts, const double* rest_xyz
     sim->seg_coarse = coarse_ok;
     if (!coarse_ok) sim->seg_ainv_h.clear();
   }
-  sim->pcg_cl = !sim->pcg_seg && ((kern == 3) || (kern == 0 && cl_fits && (many || !rr_fits)));
-  const bool df = !sim->pcg_cl && !sim->pcg_seg && ((kern == 5) || (kern == 0 && !many && df_fits));
+  const bool df = kern == 5 || (kern == 0 && team.fits);
+  sim->pcg_cl = !sim->pcg_seg && !df && ((kern == 3) || (kern == 0 && cl_fits && (many || !rr_fits)));
   sim->pcg_rr = !df && !sim->pcg_cl && !sim->pcg_seg && ((kern == 2) || (kern == 0 && rr_fits));
   sim->pcg_variant = df ? 5 : sim->pcg_rr ? 2 : 1;
+  if (!df) team = TeamHost{};
   sim->cl_rows_cap = cap;
   sim->pcg_clusters = std::max(1, std::min(max_clusters, sim->n_robots));
   if (sim->pcg_seg) {
     // partials buffer is sized by pcg_grid (already >= seg_blocks)
   } else if (sim->pcg_variant == 5) {
-    sim->pcg_grid = std::max(1, (n_free + R_df - 1) / R_df);
+    sim->pcg_grid = team.grid;
   } else if (sim->pcg_rr) {
     sim->pcg_grid = std::max(1, (n_free + PCG_RR_THREADS - 1) / PCG_RR_THREADS);
   } else {

@@ -1115,7 +1115,10 @@ __device__ void spring_update_vertex(const Dev<T>& d, int qi, int& active_out, u
       d.sp.target[3 * qi + 2] = tgt.z;
       d.spring_c[v] = R4<double>{tgt.x, tgt.y, tgt.z, active ? 1.0 : 0.0};
       active_out += active;
-      if (active) ssig += spring_term(qi, kind, face);
+      if (active) {
+        ssig += spring_term(qi, kind, face);
+        if (d.tm_springs) atomicAdd(&d.tm_springs[d.robot_of_vert ? d.robot_of_vert[v] : 0], 1);
+      }
     }
   }
 }
@@ -1174,6 +1177,7 @@ __global__ void __launch_bounds__(CAST_THREADS) k_cast(Dev<T> d) {
       d.sp.target[3 * qi + 2] = tgt.z;
       d.spring_c[v] = R4<double>{tgt.x, tgt.y, tgt.z, active ? 1.0 : 0.0};
       active_out += active;
+      if (active && d.tm_springs) atomicAdd(&d.tm_springs[rv], 1);
       if (active && d.stats) atomicAdd(&(d.hist + (d.ctrl->iter % d.hist_cap))->spring_sig, spring_term(qi, 3, f));
     }
   }
@@ -1263,6 +1267,7 @@ __global__ void __launch_bounds__(CAST_THREADS) k_cast_bvh(Dev<T> d) {
     d.sp.target[3 * qi + 2] = tgt.z;
     d.spring_c[v] = R4<double>{tgt.x, tgt.y, tgt.z, active ? 1.0 : 0.0};
     active_out += active;
+    if (active && d.tm_springs) atomicAdd(&d.tm_springs[rv], 1);
     if (active && d.stats) atomicAdd(&(d.hist + (d.ctrl->iter % d.hist_cap))->spring_sig, spring_term(qi, 3, bf));
   }
   const int ns = block_sum_int(active_out, shi);

@@ -112,6 +112,14 @@ struct BvhDev {
   const int* root;     // per robot: root code of its tree (null: one tree rooted at node 0)
 };
 
+// One part of a robot's rows in the team PCG (team.cu).
+struct TeamPart {
+  int robot, p0, np;   // the robot, its first part and how many it has
+  int row0, nrow;      // free rows
+  int halo0, n_other;  // its other parts' rows in tm_halo
+  long long ainv;      // its four rows of the robot's coarse inverse in tm_ainv
+};
+
 struct SpringDev {
   int* active;           // n_q
   int* kind;             // n_q: 0 self, 1 sphere obstacle, 2 tetrahedral obstacle
@@ -149,21 +157,30 @@ struct Dev {
   R4<T>* s;
   R4<T>* w;
   R4<T>* dx;             // PCG correction (streaming kernel)
-  R4<T>* xstep;          // dataflow PCG of an outer iteration: x_i - x_(i-1) per free row; the solve starts
+  R4<T>* xstep;          // team and batch PCG of an outer iteration: x_i - x_(i-1) per free row; the solve starts
                          //   from x_i + xstep instead of x_i (null: from x_i)
   double* partials;      // 2 x 4 x pcg grid
-  unsigned long long* df_u;  // dataflow PCG: 2 x n_free x 2 epoch-tagged words of u
-  unsigned long long* df_p;  // dataflow PCG: 2 x (grid + 1) x 4 epoch-tagged partial words
-  const int* halo_ptr;   // dataflow PCG: per block, start of its halo in halo_rows
-  const int* halo_rows;  //   distinct rows each block's SpMV reads: its own rows, then the
-                         //   others (each part ascending)
-  const int* halo_own;   //   per block, how many of its halo rows are its own
-  const int* halo_self;  //   per free row, its index in its block's halo (-1: not read)
-  const int* sl_lcol;    //   per sliced-ELL entry: the column's index in its block's halo
-  int halo_max;          //   longest halo (rows)
-  int df_rows;           //   rows (threads) per block: 288 or 384
-  const float* cg_ainv;  // dataflow PCG coarse correction: A_c^-1 (n_agg x n_agg, row-major)
-  int n_agg;             //   aggregates of 128 consecutive free rows; 0 = Jacobi only
+  // team PCG (team.cu)
+  const TeamPart* tm_part;   // parts, robot by robot
+  int tm_parts, tm_grid, tm_threads;
+  int tm_r_per, tm_row_threads;  // rows per thread, threads that have rows (FP64: per column)
+  int tm_smem, tm_ainv_off, tm_val_off, tm_lcol_off;  // dynamic shared memory: bytes, offsets
+  bool tm_cluster;           // the team is one thread-block cluster
+  int tm_coarse;             // 1: two-level preconditioner
+  int tm_levels;             //   how many of its inverses are in use
+  int tm_halo_max;           // longest halo (rows)
+  const int* tm_halo;        // per part: the rows of other parts that its rows read, ascending
+  const unsigned short* tm_lcol;  // per sliced-ELL entry: the column's index in its part's halo
+  const float4* tm_z;        // per free row: the coarse basis functions of its part
+  const float* tm_ainv;      // (A_c + sigma I)^-1 per level and robot, row-major
+  size_t tm_ainv_level;      //   floats of one level
+  int* tm_springs;           // per robot: active springs of this iteration
+  unsigned long long* tm_u;  // epoch-tagged words: 2 x n_free rows of u,
+  unsigned long long* tm_slot;  //   the reduction slots,
+  unsigned* tm_count;        //   and the teams' arrival counters, 128 bytes apart (one allocation)
+  size_t tm_zero_bytes;      //   its length
+  R4<double>* tm_b;          // 32 bytes per free row: right-hand side without the springs
+  R4<double>* tm_r;          //   and the first residual with it
   // collision
   const int* q_verts;    // n_q internal vertex ids, in ascending caller id
   const int* qf_ptr;     // n_q + 1 incident boundary faces
@@ -197,7 +214,7 @@ struct Dev {
   double k_spring, eps, cell, inv_cell, tol2;
   int max_iter, collision, stats;
   int local_threads, rhs_threads, narrow_threads;  // launch shapes (autotuned)
-  int rhs_in_pcg;        // 1: the dataflow PCG forms b, the diagonal and the iteration's record itself
+  int rhs_in_pcg;        // team PCG: 1 an outer iteration's solve, 0 the reverse pass (b and the diagonal given)
   int n_robots;          // independent systems (robots) in the mesh
   const int* robot_row;  // n_robots + 1: first free row of each robot
   int cl_rows_cap;       // rows per CTA the cluster PCG's shared memory holds

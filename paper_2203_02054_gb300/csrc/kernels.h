@@ -25,10 +25,17 @@ static constexpr int PCG_RR_MAXW = 16;   // widest sliced-ELL row kept in regist
 static constexpr int PCG_CL_THREADS = 1024;
 static constexpr int PCG_SEG_THREADS = 256;
 static constexpr int PCG_SEG_AGG_MAX = 64;  // aggregates per block of the segmented PCG's coarse correction
-static constexpr int PCG_DF_THREADS = 384;     // rows (threads) per block of the dataflow PCG
-static constexpr int PCG_DF_ROWS_SMALL = 288;  // the same with 9 warps, for systems that fit 152 such blocks
-static constexpr int PCG_DF_REPLICAS = 4;  // copies of the dataflow PCG's reduction slots
-static constexpr size_t PCG_DF_HALO_MAX_BYTES = 160 * 1024;  // halo words in shared memory
+static constexpr int TEAM_MAX_WIDTH = 16;   // team PCG: widest sliced-ELL row
+static constexpr int TEAM_MAX_PARTS = 160;  //   parts of one robot
+static constexpr int TEAM_CLUSTER = 16;     //   up to this many run as one thread-block cluster
+static constexpr int TEAM_COPIES = 4;       //   copies of the reduction slots of large teams
+static constexpr int TEAM_NT_1 = 384;       //   threads per block: one FP32 row per thread,
+static constexpr int TEAM_NT_3 = 512;       //   three FP32 rows per thread,
+static constexpr int TEAM_NT_F64 = 384;     //   one FP64 column of up to three rows per thread
+static constexpr int TEAM_LEVELS = 6;        //   inverses of the coarse matrix: for no springs,
+static constexpr float TEAM_SIGMA_1 = 1.0f / 1024;  //   springs per row of the next one (then a factor 4 each)
+static constexpr int TEAM_CONSTANTS_MAX = 4096; //   MIXED robots up to this many rows: constant basis functions alone
+static constexpr size_t TEAM_SMEM_MAX = 216 * 1024;  //   dynamic shared memory
 static constexpr int PCG_CL_SIZE = 16;   // CTAs per cluster (non-portable size)
 
 template <typename T>
@@ -45,8 +52,19 @@ template <typename T>
 cudaError_t launch_pcg(const Dev<T>& d, int grid, int variant, cudaStream_t st);
 template <typename T>
 int pcg_rr_max_rows();
-int pcg_df_max_rows(int rows);
-bool pcg_df_prepare(int rows, int smem_bytes);
+template <typename T>
+void launch_team_rhs(const Dev<T>& d, cudaStream_t st);
+template <typename T>
+cudaError_t launch_team_clear(const Dev<T>& d, cudaStream_t st);
+template <typename T>
+cudaError_t launch_pcg_team(const Dev<T>& d, cudaStream_t st);
+bool team_prepare(bool fp64, int r, bool cluster, int grid, int threads, size_t smem);
+size_t team_words(bool fp64, int n_free, int parts, int robots, size_t& slot_off, size_t& count_off);
+size_t team_smem(bool fp64, int rows, int r, int halo_max, int max_np, bool coarse, int max_width,
+                 int& ainv_off, int& val_off, int& lcol_off);
+void launch_shift(double* A, const long long* off, const int* dim, int n_mat, double sigma, cudaStream_t st);
+void launch_invert(double* A, const long long* off, const int* dim, int n_mat, int max_dim, double* C, double* D,
+                   float* out, int* bad, cudaStream_t st);
 template <typename T>
 int pcg_seg_max_blocks();
 template <typename T>
