@@ -760,6 +760,24 @@ __device__ __forceinline__ void warp_argmin(int& f, double& key, double& b1, dou
   }
 }
 
+// The same over the eight lanes of a team (all lanes of the warp take part).
+__device__ __forceinline__ void team_argmin(int& f, double& key, double& b1, double& b2) {
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) {
+    const int of = __shfl_xor_sync(0xffffffffu, f, o);
+    const double ok = __shfl_xor_sync(0xffffffffu, key, o);
+    const double o1 = __shfl_xor_sync(0xffffffffu, b1, o);
+    const double o2 = __shfl_xor_sync(0xffffffffu, b2, o);
+    const unsigned long long kb = key_bits(key), okb = key_bits(ok);
+    if (of >= 0 && (f < 0 || okb < kb || (okb == kb && of < f))) {
+      f = of;
+      key = ok;
+      b1 = o1;
+      b2 = o2;
+    }
+  }
+}
+
 // Closest-point candidate of face f for point o (lane-local running minimum).
 template <typename T>
 __device__ __forceinline__ void closest_candidate(const Dev<T>& d, int v, int rv, int f, V3 o, int& lf, double& ld,
@@ -781,111 +799,17 @@ __device__ __forceinline__ void closest_candidate(const Dev<T>& d, int v, int rv
   }
 }
 
-// Self-collision correspondence of vertex v: first exit-face hit along dir,
-// by one warp.  Every lane walks the same cells (3D-DDA); the faces listed in
-// a cell are split over the lanes and the cell's first hit is the warp
-// minimum of (t, face id), merged into the running first hit.  The result is
-// the same as a serial walk's.
+// Closest boundary face, among those not containing vertex v, to point o of v
+// (robot rv) by one warp, and the closest point's barycentrics.
 template <typename T>
-__device__ int ray_cast_warp(const Dev<T>& d, int v, int rv, V3 o, V3 dir, double& rb1, double& rb2,
-                             int& fell_back) {
+__device__ int closest_face_warp(const Dev<T>& d, int v, int rv, V3 o, double& rb1, double& rb2) {
   const int lane = threadIdx.x & 31;
-  fell_back = 0;
   int best_f = -1;
-  double best_t = 0.0;
-  unsigned long long best_lim = 0;  // bits of best_t (1 + 1e-9)
   rb1 = rb2 = 0.0;
-  // DDA set-up: lane a < 3 forms axis a's start cell, step, first boundary
-  // parameter and increment, and its bound on the ray parameter from the
-  // bounding box of this iteration's boundary faces (the ray can meet no face
-  // beyond it); the warp shares them by shuffles, so the FP64 divisions run once per
-  // axis, not once per lane.  tbox is the minimum over the axes.
-  int cell[3], step[3];
-  double tmax[3], tdel[3], tbox;
-  {
-    const int a = lane < 3 ? lane : 0;
-    const double dva = a == 0 ? dir.x : a == 1 ? dir.y : dir.z;
-    const double ova = a == 0 ? o.x : a == 1 ? o.y : o.z;
-    int c_a = 0, st_a = 0;
-    double tm_a = INFINITY, td_a = INFINITY, tb_a = INFINITY;
-    if (lane < 3) {
-      c_a = cell_coord(ova, d.inv_cell);
-      const double blo = order_decode(d.ctrl->box_lo[a]) - d.cell, bhi = order_decode(d.ctrl->box_hi[a]) + d.cell;
-      if (dva > 0.0) {
-        st_a = 1;
-        tm_a = ((c_a + 1) * d.cell - ova) / dva;
-        td_a = d.cell / dva;
-        tb_a = (bhi - ova) / dva;
-      } else if (dva < 0.0) {
-        st_a = -1;
-        tm_a = (c_a * d.cell - ova) / dva;
-        td_a = -d.cell / dva;
-        tb_a = (blo - ova) / dva;
-      }
-      // ray parameters of the walk are compared by their bit patterns below,
-      // so they are made non-negative: a start within rounding of a cell face
-      // can give -0.0 or a tiny negative first boundary (either way the walk
-      // first steps across it), and the walk starts inside the faces' box
-      tm_a = tm_a > 0.0 ? tm_a : 0.0;
-      tb_a = tb_a > 0.0 ? tb_a : 0.0;
-    }
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      cell[k] = __shfl_sync(0xffffffffu, c_a, k);
-      step[k] = __shfl_sync(0xffffffffu, st_a, k);
-      tmax[k] = __shfl_sync(0xffffffffu, tm_a, k);
-      tdel[k] = __shfl_sync(0xffffffffu, td_a, k);
-    }
-    tbox = fmin(fmin(__shfl_sync(0xffffffffu, tb_a, 0), __shfl_sync(0xffffffffu, tb_a, 1)),
-                __shfl_sync(0xffffffffu, tb_a, 2));
-  }
-  for (int it = 0; it < MAX_DDA_STEPS; ++it) {
-    const unsigned h = d.H_t + (hash_cell(cell[0], cell[1], cell[2], rv) & (d.H_f - 1u));
-    const int k0 = d.cell_start[h], k1 = min(d.cell_start[h + 1], d.cap_items);
-    int lf = -1;
-    double lt = 0.0, l1 = 0.0, l2 = 0.0;
-    for (int k = k0 + lane; k < k1; k += 32) {
-      const int f = d.items[k] - d.n_t;
-      if (d.robot_of_face && d.robot_of_face[f] != rv) continue;
-      V3 q0, q1, q2;
-      int4 fv;
-      face_verts(d, f, q0, q1, q2, fv);
-      if (fv.x == v || fv.y == v || fv.z == v) continue;
-      if (!(dot(dir, cross(sub(q1, q0), sub(q2, q0))) > 0.0)) continue;
-      double t, b1, b2;
-      if (!ray_tri(o, dir, q0, q1, q2, t, b1, b2)) continue;
-      if (lf < 0 || t < lt || (t == lt && f < lf)) {
-        lf = f;
-        lt = t;
-        l1 = b1;
-        l2 = b2;
-      }
-    }
-    if (__any_sync(0xffffffffu, lf >= 0)) {
-      warp_argmin(lf, lt, l1, l2);
-      if (best_f < 0 || key_bits(lt) < key_bits(best_t) || (lt == best_t && lf < best_f)) {
-        best_f = lf;
-        best_t = lt;
-        rb1 = l1;
-        rb2 = l2;
-        best_lim = key_bits(best_t * (1.0 + 1e-9));
-      }
-    }
-    const unsigned long long m0 = key_bits(tmax[0]), m1 = key_bits(tmax[1]), m2 = key_bits(tmax[2]);
-    const unsigned long long texit = m0 < m1 ? (m0 < m2 ? m0 : m2) : (m1 < m2 ? m1 : m2);
-    if (best_f >= 0 && best_lim < texit) return best_f;
-    if (texit >= key_bits(INFINITY) || texit > key_bits(tbox)) break;
-    const int a = (m0 <= m1 && m0 <= m2) ? 0 : (m1 <= m2 ? 1 : 2);
-    cell[a] += step[a];
-    tmax[a] += tdel[a];
-  }
-  if (best_f >= 0) return best_f;
-  fell_back = 1;
-  // No exit face hit: the closest point over the boundary faces not
-  // containing v, found by scanning cubic shells of cells around v's cell
-  // (the cells of a shell split over the lanes).  After shell k every face
-  // with a point within k cells has been seen, so the search stops once the
-  // best distance is at most k cell edges.
+  // found by scanning cubic shells of cells around v's cell (the cells of a
+  // shell split over the lanes).  After shell k every face with a point within
+  // k cells has been seen, so the search stops once the best distance is at most
+  // k cell edges.
   const int c0[3] = {cell_coord(o.x, d.inv_cell), cell_coord(o.y, d.inv_cell), cell_coord(o.z, d.inv_cell)};
   double bestd = 0.0;
   for (int k = 0; k <= 64; ++k) {
@@ -1063,10 +987,12 @@ __device__ void spring_update_vertex(const Dev<T>& d, int qi, int& active_out, u
       deferred = true;
       const int slot = atomicAdd(&d.ctrl->n_cast, 1);  // < n_q: each vertex enters once
       d.cast_list[slot] = qi;
-      const V3 n = normal();
-      d.cast_nrm[3 * qi] = n.x;
-      d.cast_nrm[3 * qi + 1] = n.y;
-      d.cast_nrm[3 * qi + 2] = n.z;
+      if (d.broad == 1) {  // (k_cast forms it itself, eight lanes per vertex)
+        const V3 n = normal();
+        d.cast_nrm[3 * qi] = n.x;
+        d.cast_nrm[3 * qi + 1] = n.y;
+        d.cast_nrm[3 * qi + 2] = n.z;
+      }
     } else if (active) {
       if (kind == 1) {
         const V3 c = {d.spheres[4 * face], d.spheres[4 * face + 1], d.spheres[4 * face + 2]};
@@ -1137,39 +1063,234 @@ __global__ void __launch_bounds__(128) k_springs(Dev<T> d) {
   narrow_block_totals(d, 0, 0, n_spr, ssig, shi);
 }
 
-// Self springs of the listed vertices: one warp per vertex shares the ray
-// cast (persistent grid, warps stride over the list); lane 0 writes the
-// spring record, v_c = hit point + eps n_f.
+// FP32 test of a face against a ray from o along the unit direction dir, which
+// may only reject what the FP64 test (exit face, then ray_tri) rejects.  The
+// signs of five triple products decide: dir.(e1 x e2) > 0 (exit face), the two
+// barycentrics and their sum, the ray parameter.  Each is formed in FP32 from
+// coordinate differences; with |dir| = 1 its rounding errors are below 8 u times
+// the product of the factors' 1-norms (u = 2^-24; two differences, dir, the
+// products and the sums), and 1e-6 = 16.8 u is used.  FP64 positions enter
+// rounded to FP32, which adds dl = 2^-22 times the coordinates' sizes to every
+// difference.  The constant covers underflow, differences above 1e9 (products
+// that could overflow) and NaN pass, like every value within its bound.
+__device__ __forceinline__ float l1(const float (&a)[3]) { return fabsf(a[0]) + fabsf(a[1]) + fabsf(a[2]); }
+__device__ __forceinline__ float triple(const float (&a)[3], const float (&b)[3], const float (&c)[3]) {
+  return a[0] * (b[1] * c[2] - b[2] * c[1]) + a[1] * (b[2] * c[0] - b[0] * c[2]) + a[2] * (b[0] * c[1] - b[1] * c[0]);
+}
+template <typename T>
+__device__ __forceinline__ bool face_may_hit(const R4<T>& q0, const R4<T>& q1, const R4<T>& q2, const float (&o)[3],
+                                             const float (&dir)[3]) {
+  const float a[3] = {(float)q0.x, (float)q0.y, (float)q0.z}, b[3] = {(float)q1.x, (float)q1.y, (float)q1.z},
+              c[3] = {(float)q2.x, (float)q2.y, (float)q2.z};
+  float e1[3], e2[3], tv[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    e1[k] = b[k] - a[k];
+    e2[k] = c[k] - a[k];
+    tv[k] = o[k] - a[k];
+  }
+  const float dl = std::is_same<T, float>::value ? 0.0f : 0x1p-22f * (l1(a) + l1(b) + l1(c) + l1(o));
+  const float n1 = l1(e1) + dl, n2 = l1(e2) + dl, n0 = l1(tv) + dl;
+  if (!(n0 + n1 + n2 < 1e9f)) return true;
+  const float tiny = 1e-25f, k = 1e-6f;
+  const float det = triple(dir, e1, e2);          // > 0 for an exit face
+  const float v1 = triple(tv, dir, e2);           // -b1 det
+  const float v2 = triple(dir, tv, e1);           // -b2 det
+  const float vt = triple(e2, tv, e1);            // -t det
+  const float bd = k * n1 * n2 + dl * (n1 + n2) + tiny, b1 = k * n0 * n2 + dl * (n0 + n2) + tiny,
+              b2 = k * n0 * n1 + dl * (n0 + n1) + tiny,
+              bt = k * n0 * n1 * n2 + dl * (n0 * n1 + n1 * n2 + n0 * n2) + tiny;
+  return !(det < -bd || v1 > b1 || v2 > b2 || -(v1 + v2) - det > bd + b1 + b2 || vt > bt);
+}
+
+// Self springs of the listed vertices: eight lanes per vertex (persistent grid,
+// the warps stride over the list four vertices at a time); v_c = hit point + eps
+// n_f.  The correspondence is the first exit-face hit of the ray from the vertex
+// along its negative area-weighted normal (3D-DDA over the face hash), the hit
+// with the smallest (t, face id); without one, the closest point.
+//
+// What bounds it is FP64: an FP64 instruction costs its scheduler 64 cycles in
+// one lane as in thirty-two, and the normal, the walk's set-up, a ray-triangle
+// test and the target are about 300 of them.  So four vertices share each of
+// those phases: a vertex's lanes take its incident faces, then its axes; the
+// teams walk their cells with the FP32 test alone until one of a cell's faces
+// passes it, and only then meet for the FP64 test of all teams' candidates.
+// Measured with k_springs, before (one warp per vertex, the FP64 test on every
+// face) and after: 395 and 133 us for the 22,400 casts of a 983,040-tet finger,
+// 82 and 53 us for the 4,300 of the gripper.
 template <typename T>
 __global__ void __launch_bounds__(CAST_THREADS) k_cast(Dev<T> d) {
   __shared__ int shi[32];
-  const int lane = threadIdx.x & 31;
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, tl = lane & 7;
+  const unsigned tmask = 0xFFu << (lane & 24);
   const int n_warps = gridDim.x * (CAST_THREADS / 32);
   const int n_cast = d.ctrl->n_cast;
   int active_out = 0;
-  for (int j = (int)((blockIdx.x * (unsigned)CAST_THREADS + threadIdx.x) >> 5); j < n_cast; j += n_warps) {
-    const int qi = chk_idx(d.ctrl, d.cast_list[j], d.n_q);
+  for (int j0 = 4 * (int)((blockIdx.x * (unsigned)CAST_THREADS + threadIdx.x) >> 5); j0 < n_cast; j0 += 4 * n_warps) {
+    const int j = j0 + (lane >> 3);
+    const bool valid = j < n_cast;
+    const int qi = valid ? chk_idx(d.ctrl, d.cast_list[j], d.n_q) : 0;
     const int v = d.q_verts[qi];
-    const V3 x = pos(d, v);
-    const V3 n = {d.cast_nrm[3 * qi], d.cast_nrm[3 * qi + 1], d.cast_nrm[3 * qi + 2]};
     const int rv = d.robot_of_vert ? d.robot_of_vert[v] : 0;
-    double b1, b2;
-    int fell_back;
-    const int f = ray_cast_warp(d, v, rv, x, scl(-1.0, n), b1, b2, fell_back);
-    if (lane == 0) {
+    const R4<T> xv = d.X[v];
+    const V3 o = {(double)xv.x, (double)xv.y, (double)xv.z};
+    // area-weighted unit normal of the incident boundary faces, summed in their
+    // listed order
+    V3 n = {0.0, 0.0, 0.0};
+    const int f0 = d.qf_ptr[qi], nf = d.qf_ptr[qi + 1] - f0, most = __reduce_max_sync(FULL, nf);
+    for (int k = 0; k < most; k += 8) {
+      V3 c = {0.0, 0.0, 0.0};
+      if (k + tl < nf) {
+        V3 q0, q1, q2;
+        int4 fv;
+        face_verts(d, d.qf[f0 + k + tl], q0, q1, q2, fv);
+        c = cross(sub(q1, q0), sub(q2, q0));
+      }
+      for (int s = 0; s < min(8, most - k); ++s)
+        n = add(n, V3{__shfl_sync(FULL, c.x, s, 8), __shfl_sync(FULL, c.y, s, 8), __shfl_sync(FULL, c.z, s, 8)});
+    }
+    const double nl = norm(n);
+    const V3 dir = nl > 0.0 ? scl(-1.0 / nl, n) : V3{0.0, 0.0, 0.0};
+    const float of[3] = {(float)xv.x, (float)xv.y, (float)xv.z};
+    const float df[3] = {(float)dir.x, (float)dir.y, (float)dir.z};
+    // DDA set-up: lane a < 3 of the team forms axis a's start cell, step, first
+    // boundary parameter and increment, and its bound on the ray parameter from
+    // the bounding box of this iteration's boundary faces (the ray can meet no
+    // face beyond it)
+    int cell[3], step[3];
+    double tmax[3], tdel[3], tbox;
+    {
+      const double dva = tl == 0 ? dir.x : tl == 1 ? dir.y : dir.z;
+      const double ova = tl == 0 ? o.x : tl == 1 ? o.y : o.z;
+      int c_a = 0, st_a = 0;
+      double tm_a = INFINITY, td_a = INFINITY, tb_a = INFINITY;
+      if (tl < 3) {
+        c_a = cell_coord(ova, d.inv_cell);
+        if (dva > 0.0 || dva < 0.0) {
+          const bool up = dva > 0.0;
+          const double bound = up ? order_decode(d.ctrl->box_hi[tl]) + d.cell : order_decode(d.ctrl->box_lo[tl]) - d.cell;
+          st_a = up ? 1 : -1;
+          tm_a = ((up ? c_a + 1 : c_a) * d.cell - ova) / dva;
+          td_a = (up ? d.cell : -d.cell) / dva;
+          tb_a = (bound - ova) / dva;
+        }
+        // ray parameters of the walk are compared by their bit patterns below,
+        // so they are made non-negative: a start within rounding of a cell face
+        // can give -0.0 or a tiny negative first boundary (either way the walk
+        // first steps across it), and the walk starts inside the faces' box
+        tm_a = tm_a > 0.0 ? tm_a : 0.0;
+        tb_a = tb_a > 0.0 ? tb_a : 0.0;
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        cell[k] = __shfl_sync(FULL, c_a, k, 8);
+        step[k] = __shfl_sync(FULL, st_a, k, 8);
+        tmax[k] = __shfl_sync(FULL, tm_a, k, 8);
+        tdel[k] = __shfl_sync(FULL, td_a, k, 8);
+      }
+      const unsigned long long t0 = key_bits(__shfl_sync(FULL, tb_a, 0, 8)), t1 = key_bits(__shfl_sync(FULL, tb_a, 1, 8)),
+                               t2 = key_bits(__shfl_sync(FULL, tb_a, 2, 8));
+      tbox = __longlong_as_double((long long)min(t0, min(t1, t2)));
+    }
+    int best_f = -1;
+    double best_t = 0.0, b1 = 0.0, b2 = 0.0;
+    unsigned long long best_lim = 0;  // bits of best_t (1 + 1e-9)
+    bool walking = valid;             // team-uniform, like the walk's whole state
+    int steps = 0, kk = 0, k1 = 0;    // cells left behind; the next entry of this cell and its end
+    auto enter = [&]() {
+      const unsigned h = d.H_t + (hash_cell(cell[0], cell[1], cell[2], rv) & (d.H_f - 1u));
+      kk = d.cell_start[h];
+      k1 = min(d.cell_start[h + 1], d.cap_items);
+    };
+    if (walking) enter();
+    while (__any_sync(FULL, walking)) {
+      // each team on its own, FP32 only, until eight entries hold a candidate
+      int cand = -1;
+      while (walking) {
+        if (kk < k1) {
+          const int k = kk + tl;
+          if (k < k1) {
+            const int f = d.items[k] - d.n_t;
+            if (!d.robot_of_face || d.robot_of_face[f] == rv) {
+              const int4 fv = chk_face(d.ctrl, d.faces[chk_idx(d.ctrl, f, d.n_f)], d.n_v);
+              if (fv.x != v && fv.y != v && fv.z != v && face_may_hit(d.X[fv.x], d.X[fv.y], d.X[fv.z], of, df)) cand = f;
+            }
+          }
+          kk += 8;
+          if (__any_sync(tmask, cand >= 0)) break;
+          continue;
+        }
+        // the cell is done
+        const unsigned long long m0 = key_bits(tmax[0]), m1 = key_bits(tmax[1]), m2 = key_bits(tmax[2]);
+        const unsigned long long texit = m0 < m1 ? (m0 < m2 ? m0 : m2) : (m1 < m2 ? m1 : m2);
+        if ((best_f >= 0 && best_lim < texit) || texit >= key_bits(INFINITY) || texit > key_bits(tbox) ||
+            ++steps >= MAX_DDA_STEPS) {
+          walking = false;
+          break;
+        }
+        if (m0 <= m1 && m0 <= m2) {
+          cell[0] += step[0];
+          tmax[0] += tdel[0];
+        } else if (m1 <= m2) {
+          cell[1] += step[1];
+          tmax[1] += tdel[1];
+        } else {
+          cell[2] += step[2];
+          tmax[2] += tdel[2];
+        }
+        enter();
+      }
+      __syncwarp();
+      // all teams' candidates, FP64
+      int lf = -1;
+      double lt = 0.0, l1 = 0.0, l2 = 0.0;
+      if (cand >= 0) {
+        V3 q0, q1, q2;
+        int4 fv;
+        face_verts(d, cand, q0, q1, q2, fv);
+        if (dot(dir, cross(sub(q1, q0), sub(q2, q0))) > 0.0 && ray_tri(o, dir, q0, q1, q2, lt, l1, l2)) lf = cand;
+      }
+      if (__any_sync(FULL, lf >= 0)) {
+        team_argmin(lf, lt, l1, l2);
+        if (lf >= 0 && (best_f < 0 || key_bits(lt) < key_bits(best_t) || (lt == best_t && lf < best_f))) {
+          best_f = lf;
+          best_t = lt;
+          b1 = l1;
+          b2 = l2;
+          best_lim = key_bits(best_t * (1.0 + 1e-9));
+        }
+      }
+    }
+    // vertices without a hit, one after the other by the whole warp
+    const bool missed = valid && best_f < 0;
+    unsigned todo = __ballot_sync(FULL, missed && tl == 0);
+    while (todo) {
+      const int src = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const V3 os = {__shfl_sync(FULL, o.x, src), __shfl_sync(FULL, o.y, src), __shfl_sync(FULL, o.z, src)};
+      double c1, c2;
+      const int f = closest_face_warp(d, __shfl_sync(FULL, v, src), __shfl_sync(FULL, rv, src), os, c1, c2);
+      if ((lane & 24) == (src & 24)) {
+        best_f = f;
+        b1 = c1;
+        b2 = c2;
+      }
+    }
+    if (valid && tl == 0) {
       V3 tgt = {0.0, 0.0, 0.0};
-      if (f >= 0) {
-        V3 nf;
-        const V3 bp = face_point(d, f, b1, b2, nf);
-        tgt = add(bp, scl(d.eps, nf));
+      if (best_f >= 0) {
+        V3 nh;
+        const V3 bp = face_point(d, best_f, b1, b2, nh);
+        tgt = add(bp, scl(d.eps, nh));
       } else {
         b1 = b2 = 0.0;
       }
-      const int active = f >= 0;
+      const int active = best_f >= 0;
       d.sp.active[qi] = active;
-      d.sp.fallback[qi] = fell_back;
+      d.sp.fallback[qi] = missed;
       d.sp.kind[qi] = 0;
-      d.sp.face[qi] = f;
+      d.sp.face[qi] = best_f;
       d.sp.bary[2 * qi] = b1;
       d.sp.bary[2 * qi + 1] = b2;
       d.sp.target[3 * qi] = tgt.x;
@@ -1178,7 +1299,8 @@ __global__ void __launch_bounds__(CAST_THREADS) k_cast(Dev<T> d) {
       d.spring_c[v] = R4<double>{tgt.x, tgt.y, tgt.z, active ? 1.0 : 0.0};
       active_out += active;
       if (active && d.tm_springs) atomicAdd(&d.tm_springs[rv], 1);
-      if (active && d.stats) atomicAdd(&(d.hist + (d.ctrl->iter % d.hist_cap))->spring_sig, spring_term(qi, 3, f));
+      if (active && d.stats)
+        atomicAdd(&(d.hist + (d.ctrl->iter % d.hist_cap))->spring_sig, spring_term(qi, 3, best_f));
     }
   }
   const int ns = block_sum_int(active_out, shi);
@@ -1330,12 +1452,12 @@ template <typename T>
 void launch_springs(const Dev<T>& d, cudaStream_t st) {
   if (d.n_q <= 0) return;
   if (d.broad != 1) k_springs<T><<<(d.n_q + 127) / 128, 128, 0, st>>>(d);
-  // enough warps for one pass over a list of up to 8,192 casts
+  // enough teams for one pass over a list of up to 32,768 casts
   if (d.broad == 1) {
     k_cast_bvh<T><<<std::min((d.n_q + CAST_THREADS - 1) / CAST_THREADS, 1024), CAST_THREADS, 0, st>>>(d);
     return;
   }
-  const int per_block = CAST_THREADS / 32;
+  const int per_block = CAST_THREADS / 8;
   const int blocks = std::min((d.n_q + per_block - 1) / per_block, 1024);
   k_cast<T><<<blocks, CAST_THREADS, 0, st>>>(d);
 }
