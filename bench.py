@@ -545,9 +545,9 @@ def main():
     units = float(m.n_tets) * n_iters * args.steps * world
     value, ms_max = aggregate(ms, float(m.n_tets) * n_iters * args.steps, pg, "cuda")
     stats = casim.casim_get_stats(sim.h)
-    # 2 hash binning + 1 single-pass scan + narrow phase + spring update + ray casts + local step + RHS gather + PCG; the
+    # query vertices + 3 of the faces' hash + narrow phase + spring update + ray casts + local step + RHS gather + PCG; the
     # team PCG (kernel 5) finalizes the iteration itself, the others need 1 launch more
-    kernels_per_iter = 9 if stats.pcg_kernel == 5 else 10
+    kernels_per_iter = 10 if stats.pcg_kernel == 5 else 11
     gpu_launches = kernels_per_iter * n_iters * args.steps
     hist = casim.casim_get_history(sim.h, n_iters)
 

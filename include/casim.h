@@ -131,7 +131,7 @@ typedef struct {
   int32_t local_block;      /* launch shapes (threads per block; 0 = default):   */
   int32_t rhs_block;        /*   local step 64/128/256 (128), RHS gather          */
   int32_t narrow_block;     /*   128/256/512 (256), narrow phase 128/256/512 (256,
-                               one warp per query vertex).  Results do not depend
+                               one thread per tet; 512 runs as 256).  Results do not depend
                                on them except for the summation order of the
                                energy statistic; the autotuner picks them        */
   int32_t pcg_block;        /* free vertices per block of the team PCG (5) in MIXED:
@@ -371,7 +371,7 @@ int casim_get_phase_times(casim_sim* sim, double* ms_out5);
    Computes the self-collision pairs of Eq. 3 exactly as a casim_step
    iteration does (spatial hash + exact strict point-in-tet test), for
    positions given by the caller, without allocating: all intermediate data
-   lives in one static device array of about 6.2 MiB that every GPU which
+   lives in one static device array of about 2.2 MiB that every GPU which
    loads the library holds until the process exits.
      n_verts, dev_xyz   device, n_verts*3 floats, vertex positions
      n_tets, dev_tets   device, n_tets*4 int32 vertex ids (16-byte aligned),

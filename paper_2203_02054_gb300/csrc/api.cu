@@ -255,8 +255,14 @@ struct casim_sim {
   cudaStream_t cap_stream = nullptr;
   // graph capture only: the local step's branch, forked from and joined back
   // into cap_stream
-  cudaStream_t side_stream = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  cudaStream_t side_stream = nullptr, face_stream = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_cleared = nullptr, ev_faces = nullptr;
+  void destroy_streams() {
+    for (cudaStream_t* s : {&cap_stream, &side_stream, &face_stream})
+      if (*s) cudaStreamDestroy(*s), *s = nullptr;
+    for (cudaEvent_t* e : {&ev_fork, &ev_join, &ev_cleared, &ev_faces})
+      if (*e) cudaEventDestroy(*e), *e = nullptr;
+  }
   std::string err;
   int device = 0;
   bool has_mesh = false;
@@ -283,7 +289,11 @@ struct casim_sim {
   int4 *tet = nullptr, *faces = nullptr;
   int *inc_ptr = nullptr, *inc = nullptr, *sl_ptr = nullptr, *sl_col = nullptr;
   int *q_verts_d = nullptr, *qf_ptr = nullptr, *qf = nullptr;
-  int *cell_count = nullptr, *cell_start = nullptr, *cell_cursor = nullptr, *items = nullptr;
+  int *q_head = nullptr, *q_next = nullptr, *cell_count = nullptr, *cell_total = nullptr, *items = nullptr;
+  unsigned* q_bits = nullptr;
+  unsigned long long* entries = nullptr;
+  float4* q_pos = nullptr;
+  int2* cell_range = nullptr;
   int *pair_count = nullptr, *pair_tet = nullptr, *obs_sphere = nullptr, *int_of_user_d = nullptr;
   int* cast_list = nullptr;
   double* cast_nrm = nullptr;
@@ -294,7 +304,7 @@ struct casim_sim {
   IterRec* hist = nullptr;
   int hist_cap = 4096;
   CollisionScratch cs{};
-  unsigned H_t = 0, H_f = 0;
+  unsigned H_q = 0, H_f = 0;
   int cap_items = 0, n_slices = 0, pcg_grid = 1, n_e_local = 0, n_e_spring = 0;
   bool pcg_rr = false;  // register-resident PCG (one row per thread)
   bool pcg_cl = false;  // cluster PCG (one cluster per robot, work queue)
@@ -492,11 +502,16 @@ Dev<T> make_dev(casim_sim* sim) {
   d.faces = sim->faces;
   d.spheres = sim->spheres_d;
   d.spheres_f = sim->spheres_fd;
-  d.H_t = sim->H_t;
+  d.H_q = sim->H_q;
   d.H_f = sim->H_f;
+  d.q_head = sim->q_head;
+  d.q_bits = sim->q_bits;
+  d.q_next = sim->q_next;
+  d.q_pos = sim->q_pos;
   d.cell_count = sim->cell_count;
-  d.cell_start = sim->cell_start;
-  d.cell_cursor = sim->cell_cursor;
+  d.cell_total = sim->cell_total;
+  d.cell_range = sim->cell_range;
+  d.entries = sim->entries;
   d.items = sim->items;
   d.cap_items = sim->cap_items;
   d.pair_count = sim->pair_count;
@@ -604,14 +619,16 @@ cudaError_t upload_spheres(casim_sim* sim) {
 }
 
 // Enqueues one outer iteration on stream st (used for graph capture and for
-// the timed eager path).  With a side stream (graph capture) the local step
-// runs on it, concurrently with the spring update and the ray casts: it
-// reads only the positions, which no collision kernel writes, and writes
-// only the projections P and its energy partials, which the collision
-// kernels do not read; the iteration's record takes both sides' terms by
-// integer atomics.  The part of the team PCG's right-hand side that does not
-// depend on the springs and the clearing of its words follow it on that
-// branch.  The global solve waits for both branches.
+// the timed eager path).  With graph capture two more branches run beside the
+// collision check and the spring update.
+// The local step reads only the positions, which no collision kernel writes,
+// and writes only the projections P and its energy partials, which the
+// collision kernels do not read; the iteration's record takes both sides' terms
+// by integer atomics.  The part of the team PCG's right-hand side that does not
+// depend on the springs and the clearing of its words are on that branch, and
+// the global solve waits for it.
+// The faces' side of the broad phase (hash or tree) is read by the ray casts
+// alone, and these wait for it.
 // NVTX range for profilers (a no-op unless a tool is attached); in graph
 // replay the ranges mark the capture, in eager mode every iteration.
 struct NvtxRange {
@@ -620,21 +637,18 @@ struct NvtxRange {
 };
 
 template <typename T>
-cudaError_t enqueue_iteration(casim_sim* sim, cudaStream_t st, cudaEvent_t* ev, cudaStream_t side = nullptr) {
+cudaError_t enqueue_iteration(casim_sim* sim, cudaStream_t st, cudaEvent_t* ev, bool branches = false) {
   NvtxRange outer("casim iteration");
   const Dev<T> d = make_dev<T>(sim);
   // the team PCG: its right-hand side is gathered beside the spring update,
   // and with one robot it writes the iteration's record itself
   const bool team = sim->pcg_variant == 5;
   if (ev) cudaEventRecord(ev[0], st);
-  if (d.collision >= 1 && d.n_q > 0) {
-    NvtxRange r("collision check");
-    launch_collision<T>(d, sim->cs, st);
-  }
-  if (ev) cudaEventRecord(ev[1], st);
   Dev<T> dp = d;
   dp.rhs_in_pcg = team ? 1 : 0;
   dp.xstep = (team || sim->pcg_seg) ? (R4<T>*)sim->xstep : nullptr;
+  const bool contact = d.collision >= 1 && d.n_q > 0;
+  cudaStream_t side = branches ? sim->side_stream : nullptr;
   if (side) {
     cudaEventRecord(sim->ev_fork, st);
     cudaStreamWaitEvent(side, sim->ev_fork, 0);
@@ -646,9 +660,23 @@ cudaError_t enqueue_iteration(casim_sim* sim, cudaStream_t st, cudaEvent_t* ev, 
     if (team) launch_team_rhs<T>(dp, side);
     cudaEventRecord(sim->ev_join, side);
   }
-  if (d.collision >= 1 && d.n_q > 0) {
+  if (contact) {
+    NvtxRange r("collision check");
+    launch_broad_clear<T>(d, sim->cs, st);
+    cudaStream_t fs = st;
+    if (branches) {
+      fs = sim->face_stream;
+      cudaEventRecord(sim->ev_cleared, st);
+      cudaStreamWaitEvent(fs, sim->ev_cleared, 0);
+    }
+    launch_faces<T>(d, fs);
+    if (branches) cudaEventRecord(sim->ev_faces, fs);
+    launch_collision<T>(d, st);
+  }
+  if (ev) cudaEventRecord(ev[1], st);
+  if (contact) {
     NvtxRange r("spring update");
-    launch_springs<T>(d, st);
+    launch_springs<T>(d, st, branches ? sim->ev_faces : nullptr);
   }
   if (ev) cudaEventRecord(ev[2], st);
   if (side) {
@@ -818,20 +846,22 @@ int upload_typed(casim_sim* sim, const std::vector<double>& rest_int, const std:
   sim->faces = sim->dalloc<int4>(n_f);
   sim->spheres_d = sim->dalloc<double>(4 * 64);
   sim->spheres_fd = sim->dalloc<float>(4 * 64);
-  const size_t H = (size_t)sim->H_t + sim->H_f;
-  // the count array is followed by the single-pass scan's status words and
-  // ticket (8-byte aligned), which its memset zeroes as well
-  sim->cell_count = sim->dalloc<int>(H + 1 + scan_lookback_extra_ints((int)H + 1));
   {
-    const size_t off = ((H + 1 + 1) / 2) * 2;  // ints, rounded up to 8 bytes
-    sim->cs.tile_status = reinterpret_cast<unsigned long long*>(sim->cell_count + off);
-    sim->cs.ticket = reinterpret_cast<unsigned*>(sim->cs.tile_status + (scan_tiles((int)H + 1) + 1));
+    // zeroed together each iteration: entries (2 ints) and the faces' total, the
+    // bits, the list heads, the face cells' counts
+    const size_t n = 4 + sim->H_q / 8 + (size_t)sim->H_q + sim->H_f;
+    int* p = sim->dalloc<int>(n);
+    sim->cs = {p, n * sizeof(int)};
+    sim->entries = reinterpret_cast<unsigned long long*>(p);
+    sim->cell_total = p + 2;
+    sim->q_bits = reinterpret_cast<unsigned*>(p + 4);
+    sim->q_head = p + 4 + sim->H_q / 8;
+    sim->cell_count = sim->q_head + sim->H_q;
   }
-  sim->cell_start = sim->dalloc<int>(H + 1);
-  sim->cell_cursor = sim->dalloc<int>(H);
+  sim->q_next = sim->dalloc<int>(n_q);
+  sim->q_pos = sim->dalloc<float4>(n_q);
+  sim->cell_range = sim->dalloc<int2>(sim->H_f);
   sim->items = sim->dalloc<int>(sim->cap_items);
-  sim->cs.tile_sums = sim->dalloc<int>(scan_tiles((int)H + 1) + 1);
-  sim->cs.total = sim->dalloc<int>(1);
   sim->pair_count = sim->dalloc<int>(n_q);
   sim->pair_tet = sim->dalloc<int>((size_t)n_q * sim->params.max_pairs_per_vertex);
   sim->obs_sphere = sim->dalloc<int>(n_q);
@@ -1085,7 +1115,7 @@ int capture_graph(casim_sim* sim) {
   }
   cudaGraph_t g = nullptr;
   CK(cudaStreamBeginCapture(sim->cap_stream, cudaStreamCaptureModeThreadLocal));
-  cudaError_t e = enqueue_iteration<T>(sim, sim->cap_stream, nullptr, sim->side_stream);
+  cudaError_t e = enqueue_iteration<T>(sim, sim->cap_stream, nullptr, true);
   cudaError_t e2 = cudaStreamEndCapture(sim->cap_stream, &g);
   if (e != cudaSuccess) {
     if (g) cudaGraphDestroy(g);
@@ -1226,12 +1256,13 @@ int casim_create(const casim_params* params, void* cuda_stream, casim_sim** out)
   if (cudaGetDevice(&sim->device) != cudaSuccess ||
       cudaStreamCreateWithFlags(&sim->cap_stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaStreamCreateWithFlags(&sim->side_stream, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaStreamCreateWithFlags(&sim->face_stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&sim->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&sim->ev_join, cudaEventDisableTiming) != cudaSuccess) {
+      cudaEventCreateWithFlags(&sim->ev_join, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&sim->ev_cleared, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&sim->ev_faces, cudaEventDisableTiming) != cudaSuccess) {
     g_create_error = "CUDA unavailable";
-    if (sim->cap_stream) cudaStreamDestroy(sim->cap_stream);
-    if (sim->side_stream) cudaStreamDestroy(sim->side_stream);
-    if (sim->ev_fork) cudaEventDestroy(sim->ev_fork);
+    sim->destroy_streams();
     delete sim;
     return CASIM_E_CUDA;
   }
@@ -1995,7 +2026,7 @@ static int upload_robots(casim_sim* sim, int32_t n_verts, const double* rest_xyz
     bvh_build(cen, sim->n_f, sim->robot_of_face_h.data(), n_robots, sim->bvh_f_h);
   }
   // ---- spatial hash sizes ----
-  sim->H_t = (unsigned)pow2_at_least(2 * (size_t)n_t);
+  sim->H_q = (unsigned)pow2_at_least(4 * (size_t)std::max(sim->n_q, 16));
   sim->H_f = (unsigned)pow2_at_least(2 * (size_t)std::max(sim->n_f, 1));
   sim->cap_items = (int)std::min<long long>(16LL * (n_t + sim->n_f) + 4096, 2000000000LL);
   // ---- PCG grid: co-resident blocks, no more than the rows need ----
@@ -3117,10 +3148,7 @@ void casim_destroy(casim_sim* sim) {
   if (!sim) return;
   cudaStreamSynchronize(sim->stream);
   sim->free_all();
-  if (sim->cap_stream) cudaStreamDestroy(sim->cap_stream);
-  if (sim->side_stream) cudaStreamDestroy(sim->side_stream);
-  if (sim->ev_fork) cudaEventDestroy(sim->ev_fork);
-  if (sim->ev_join) cudaEventDestroy(sim->ev_join);
+  sim->destroy_streams();
   delete sim;
 }
 

@@ -1,21 +1,21 @@
 // Collision check (Sec. II-B, Eq. 3, Eq. 4) and spring update (Sec. II-C,
 // Eq. 5, Sec. III-A.3) kernels.
 //
-// Broad phase: one spatial hash over tets and one over boundary faces, rebuilt
-// every iteration from the current positions (counting sort: count, scan,
-// fill).  A point strictly inside a tet lies in the tet's closed bounding box,
-// whose cell range covers the point's cell, so the hash never drops a pair;
-// hash collisions only add candidates.
+// Broad phase: a spatial hash of the query vertices (lists) and one of the
+// boundary faces (counting sort), rebuilt every iteration from the current
+// positions.  A point strictly inside a tet lies in the tet's closed bounding
+// box, whose cell range covers the point's cell, so a walk over the cells of
+// every tet's box meets every pair.
 //
-// Narrow phase: one warp per non-fixed boundary vertex tests the tets of its
-// cell with exact orientation signs (predicates.cuh), so the pair set equals
-// the brute-force definition bit for bit.
+// Narrow phase: one thread per tet tests the vertices listed in its cells with
+// exact orientation signs (predicates.cuh), so the pair set equals the
+// brute-force definition bit for bit.
 //
 // Spring update: one thread per non-fixed boundary vertex for obstacle
 // targets (closed form) and the paper's release condition; self-collision
 // targets by a ray cast along -n(v) (3D-DDA cell walk of Amanatides and Woo
-// 1987 over the face hash, Moller-Trumbore 1997 ray-triangle test), one warp
-// per casting vertex.  All spring geometry is evaluated in FP64.
+// 1987 over the face hash, Moller-Trumbore 1997 ray-triangle test), eight
+// lanes per casting vertex.  All spring geometry is evaluated in FP64.
 #include <algorithm>
 
 #include "bvh.cuh"
@@ -36,37 +36,24 @@ __device__ __forceinline__ void load3(const R4<T>* X, int v, double& x, double& 
   z = (double)a.z;
 }
 
-// Bounding box of item i: tets are items [0, n_t), boundary faces [n_t, n_t + n_f),
-// in the positions' own precision.
-template <typename T>
-__device__ __forceinline__ bool item_box_t(const Dev<T>& d, int i, T lo[3], T hi[3]) {
-  int vs[4];
-  int nv;
-  if (i < d.n_t) {
-    const int4 t = chk_idx4(d.ctrl, d.tet[i], d.n_v);
-    vs[0] = t.x; vs[1] = t.y; vs[2] = t.z; vs[3] = t.w;
-    nv = 4;
-  } else {
-    const int4 f = chk_face(d.ctrl, d.faces[i - d.n_t], d.n_v);
-    vs[0] = f.x; vs[1] = f.y; vs[2] = f.z;
-    nv = 3;
-  }
-  // min/max in the positions' own precision, converted once (exact)
-  const R4<T> a0 = d.X[vs[0]];
-  T l[3] = {a0.x, a0.y, a0.z}, h[3] = {a0.x, a0.y, a0.z};
-  bool ok = isfinite(a0.x) && isfinite(a0.y) && isfinite(a0.z);
-  for (int k = 1; k < nv; ++k) {
-    const R4<T> a = d.X[vs[k]];
-    const T c[3] = {a.x, a.y, a.z};
+// Bounding box of up to four corners in the positions' own precision; false if
+// one is not finite.
+template <typename T, int NV>
+__device__ __forceinline__ bool corner_box(const R4<T> (&c)[NV], T lo[3], T hi[3]) {
+  bool ok = true;
+  lo[0] = hi[0] = c[0].x;
+  lo[1] = hi[1] = c[0].y;
+  lo[2] = hi[2] = c[0].z;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    const T a[3] = {c[k].x, c[k].y, c[k].z};
+#pragma unroll
     for (int j = 0; j < 3; ++j) {
-      ok = ok && isfinite(c[j]);
-      l[j] = fmin(l[j], c[j]);
-      h[j] = fmax(h[j], c[j]);
+      ok = ok && isfinite(a[j]);
+      if (k == 0) continue;
+      lo[j] = fmin(lo[j], a[j]);
+      hi[j] = fmax(hi[j], a[j]);
     }
-  }
-  for (int j = 0; j < 3; ++j) {
-    lo[j] = l[j];
-    hi[j] = h[j];
   }
   return ok;
 }
@@ -118,41 +105,41 @@ __device__ __forceinline__ void reduce_box(Ctrl* c, bool valid, const double lo[
   }
 }
 
+// Adds one block's number of hash entries to the iteration's total; a total
+// above the declared capacity is an overflow.
+template <typename T>
+__device__ __forceinline__ void add_entries(const Dev<T>& d, unsigned long long n) {
+  if (n == 0) return;
+  if (atomicAdd(d.entries, n) + n > (unsigned long long)d.cap_items) set_status(d.ctrl, ST_OVERFLOW);
+}
+
+// ---- hash of the boundary faces: count, place the cells, fill ----
+static constexpr int FACE_THREADS = 256;
+
 template <typename T, bool FILL>
-__global__ void __launch_bounds__(256) k_grid_bin(Dev<T> d) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int n = d.n_t + d.n_f;
+__global__ void __launch_bounds__(FACE_THREADS) k_faces(Dev<T> d) {
+  const int f = blockIdx.x * FACE_THREADS + threadIdx.x;
   T lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
-  const bool ok = i < n && item_box_t(d, i, lo, hi);
-  if (!FILL) {
-    // the box of the boundary faces bounds the ray walks (no face lies beyond it)
-    const bool face = ok && i >= d.n_t;
-    double lod[3] = {0.0, 0.0, 0.0}, hid[3] = {0.0, 0.0, 0.0};
-    if (face)
-      for (int j = 0; j < 3; ++j) {
-        lod[j] = (double)lo[j];
-        hid[j] = (double)hi[j];
-      }
-    reduce_box(d.ctrl, face, lod, hid);
+  bool ok = false;
+  if (f < d.n_f) {
+    const int4 fv = chk_face(d.ctrl, d.faces[f], d.n_v);
+    const R4<T> c[3] = {d.X[fv.x], d.X[fv.y], d.X[fv.z]};
+    ok = corner_box<T, 3>(c, lo, hi);
   }
-  if (i >= n) return;
+  // (converted exactly)
+  const double lod[3] = {(double)lo[0], (double)lo[1], (double)lo[2]},
+               hid[3] = {(double)hi[0], (double)hi[1], (double)hi[2]};
+  // the box of the boundary faces bounds the ray walks (no face lies beyond it)
+  if (!FILL) reduce_box(d.ctrl, ok, lod, hid);
+  if (f >= d.n_f) return;
   if (!ok) {
     if (!FILL) set_status(d.ctrl, ST_NONFINITE);
     return;
   }
   int c0[3], c1[3];
-  const bool is_tet = i < d.n_t;
-  if (std::is_same<T, float>::value && is_tet) {
-    const float inv_f = (float)d.inv_cell;
-    for (int j = 0; j < 3; ++j) {
-      c0[j] = cell_coord_f((float)lo[j], inv_f);
-      c1[j] = cell_coord_f((float)hi[j], inv_f);
-    }
-  } else {
-    for (int j = 0; j < 3; ++j) {
-      c0[j] = cell_coord((double)lo[j], d.inv_cell);
-      c1[j] = cell_coord((double)hi[j], d.inv_cell);
-    }
+  for (int j = 0; j < 3; ++j) {
+    c0[j] = cell_coord(lod[j], d.inv_cell);
+    c1[j] = cell_coord(hid[j], d.inv_cell);
   }
   const long long ncell =
       (long long)(c1[0] - c0[0] + 1) * (c1[1] - c0[1] + 1) * (c1[2] - c0[2] + 1);
@@ -160,23 +147,21 @@ __global__ void __launch_bounds__(256) k_grid_bin(Dev<T> d) {
     if (!FILL) set_status(d.ctrl, ST_OVERFLOW);
     return;
   }
-  const unsigned base = is_tet ? 0u : d.H_t;
-  const unsigned mask = (is_tet ? d.H_t : d.H_f) - 1u;
-  const int robot = is_tet ? (d.robot_of_tet ? d.robot_of_tet[i] : 0) : (d.robot_of_face ? d.robot_of_face[i - d.n_t] : 0);
+  const int robot = d.robot_of_face ? d.robot_of_face[f] : 0;
   for (int cz = c0[2]; cz <= c1[2]; ++cz)
     for (int cy = c0[1]; cy <= c1[1]; ++cy)
       for (int cx = c0[0]; cx <= c1[0]; ++cx) {
-        const unsigned h = base + (hash_cell(cx, cy, cz, robot) & mask);
+        const unsigned h = hash_cell(cx, cy, cz, robot) & (d.H_f - 1u);
         if (!FILL) {
           atomicAdd(&d.cell_count[h], 1);
         } else {
-          const int pos = d.cell_start[h] + atomicAdd(&d.cell_cursor[h], 1);
-          if (pos < d.cap_items) d.items[pos] = i;
+          const int pos = atomicAdd(&d.cell_range[h].y, 1);
+          if (pos < d.cap_items) d.items[pos] = f;
         }
       }
 }
 
-// ---- exclusive scan of cell_count into cell_start (three small kernels) ----
+// ---- exclusive scan (three small kernels) ----
 static constexpr int SCAN_THREADS = 256;
 static constexpr int SCAN_PER_THREAD = 8;
 static constexpr int SCAN_TILE = SCAN_THREADS * SCAN_PER_THREAD;
@@ -210,7 +195,7 @@ __global__ void k_scan_tiles(const int* __restrict__ in, int* __restrict__ out, 
 }
 
 // Single block: exclusive scan of the tile sums in place, total into *total.
-__global__ void k_scan_top(int* tile_sums, int n_tiles, int* total_out, Ctrl* ctrl, int cap) {
+__global__ void k_scan_top(int* tile_sums, int n_tiles, int* total_out) {
   __shared__ int sh[1024];
   __shared__ int carry;
   if (threadIdx.x == 0) carry = 0;
@@ -231,13 +216,7 @@ __global__ void k_scan_top(int* tile_sums, int n_tiles, int* total_out, Ctrl* ct
     if (threadIdx.x == 1023) carry += sh[1023];
     __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    *total_out = carry;
-    if (ctrl) {
-      ctrl->n_items = carry;
-      if (carry > cap) atomicOr(&ctrl->status, ST_OVERFLOW);
-    }
-  }
+  if (threadIdx.x == 0) *total_out = carry;
 }
 
 __global__ void k_scan_add(int* out, const int* tile_sums, int n) {
@@ -245,112 +224,48 @@ __global__ void k_scan_add(int* out, const int* tile_sums, int n) {
   if (i < n) out[i] += tile_sums[i / SCAN_TILE];
 }
 
-// ---- single-pass exclusive scan with decoupled look-back -----------------
-// (Merrill and Garland 2016).  Each block takes a tile ticket (so every
-// smaller tile belongs to a block that is already running), scans its tile,
-// publishes the tile's sum as a status word (flag 1: the tile's own sum,
-// flag 2: the inclusive prefix up to and including the tile), and warp 0
-// walks back over the predecessors' words, 32 at a time, adding own sums
-// until it meets an inclusive prefix.  Waits for a predecessor's word are
-// bounded by the clock budget (then ST_TIMEOUT).  Integer sums, so the result
-// is the same as any other scan order.  The status words and the ticket are
-// zeroed with the count array before each use; the last tile resets nothing
-// and writes the total (with the capacity check).
-__device__ __forceinline__ unsigned long long scan_word(unsigned flag, int v) {
-  return ((unsigned long long)flag << 62) | (unsigned)v;
-}
-__device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_lookback(const int* __restrict__ in, int* __restrict__ out, int n,
-                                                                unsigned long long* status, unsigned* ticket,
-                                                                int* total_out, Ctrl* ctrl, int cap,
-                                                                unsigned long long budget) {
-  __shared__ int sh[SCAN_THREADS];
-  __shared__ int s_tile, s_prefix;
-  if (threadIdx.x == 0) s_tile = (int)atomicAdd(ticket, 1u);
-  __syncthreads();
-  const int tile = s_tile;
-  const int base = tile * SCAN_TILE + threadIdx.x * SCAN_PER_THREAD;
+// Places the face cells in the item array, (start, start) for each: the cells
+// only need disjoint ranges, in whatever order, so a block takes the range of
+// its tile with one addition to a global counter instead of waiting for the
+// tiles before it, and the fill moves the end.
+template <typename T>
+__global__ void __launch_bounds__(SCAN_THREADS) k_place_cells(Dev<T> d) {
+  __shared__ int s_warp[SCAN_THREADS / 32], s_base;
+  const int base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_PER_THREAD, n = (int)d.H_f;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   int v[SCAN_PER_THREAD];
   int s = 0;
 #pragma unroll
   for (int k = 0; k < SCAN_PER_THREAD; ++k) {
-    v[k] = (base + k < n) ? in[base + k] : 0;
+    v[k] = (base + k < n) ? d.cell_count[base + k] : 0;
     s += v[k];
   }
-  sh[threadIdx.x] = s;
-  __syncthreads();
-  for (int off = 1; off < SCAN_THREADS; off <<= 1) {
-    const int t = (threadIdx.x >= off) ? sh[threadIdx.x - off] : 0;
-    __syncthreads();
-    sh[threadIdx.x] += t;
-    __syncthreads();
-  }
-  const int agg = sh[SCAN_THREADS - 1];
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    int prefix = 0;
-    if (tile == 0) {
-      if (lane == 0) st_relaxed_u64(status + tile, scan_word(2u, agg));
-    } else {
-      if (lane == 0) st_relaxed_u64(status + tile, scan_word(1u, agg));
-      long long t0 = 0;
-      unsigned polls = 0;
-      bool failed = false;
-      for (int j = tile - 1; j >= 0 && !failed; j -= 32) {
-        const int q = j - lane;  // predecessor this lane reads (nearest first)
-        unsigned long long w = q >= 0 ? ld_relaxed_u64(status + q) : scan_word(1u, 0);
-        // wait until every word of the window is published
-        while (__any_sync(0xffffffffu, (w >> 62) == 0ull)) {
-          if ((++polls & 31u) == 0) {
-            const long long now = clock64();
-            if (t0 == 0) t0 = now;
-            else if ((unsigned long long)(now - t0) > budget) {
-              failed = true;
-              break;
-            }
-          }
-          if ((w >> 62) == 0ull) w = ld_relaxed_u64(status + q);
-        }
-        if (failed) break;
-        const unsigned incl = __ballot_sync(0xffffffffu, (w >> 62) == 2ull);
-        const int stop = incl ? __ffs(incl) - 1 : 32;  // nearest inclusive prefix in the window
-        int part = (lane <= stop && q >= 0) ? (int)(unsigned)(w & 0xFFFFFFFFull) : 0;
+  int incl = s;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
-        prefix += __shfl_sync(0xffffffffu, part, 0);
-        if (incl) break;
-      }
-      if (failed && lane == 0) atomicOr(&ctrl->status, ST_TIMEOUT);
-      if (lane == 0) st_relaxed_u64(status + tile, scan_word(2u, prefix + agg));
-    }
-    if (lane == 0) s_prefix = prefix;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  if (lane == 31) s_warp[wid] = incl;
+  __syncthreads();
+  int before = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < SCAN_THREADS / 32; ++w) {
+    if (w < wid) before += s_warp[w];
+    total += s_warp[w];
+  }
+  if (threadIdx.x == 0) {
+    s_base = total ? atomicAdd(d.cell_total, total) : 0;
+    add_entries(d, (unsigned long long)total);
   }
   __syncthreads();
-  int run = s_prefix + sh[threadIdx.x] - s;  // exclusive prefix of this thread
+  int run = s_base + before + incl - s;
 #pragma unroll
   for (int k = 0; k < SCAN_PER_THREAD; ++k) {
-    if (base + k < n) out[base + k] = run;
+    if (base + k < n) d.cell_range[base + k] = make_int2(run, run);
     run += v[k];
   }
-  if (tile == (int)gridDim.x - 1 && threadIdx.x == 0) {
-    const int tot = s_prefix + agg;
-    *total_out = tot;
-    if (ctrl) {
-      ctrl->n_items = tot;
-      if (tot > cap) atomicOr(&ctrl->status, ST_OVERFLOW);
-    }
-  }
 }
-
-int scan_lookback_extra_ints(int n) { return 2 + 2 * (scan_tiles(n) + 1) + 2; }
 
 // ---- narrow phase ----
 __device__ __forceinline__ int orient_t(float ax, float ay, float az, float bx, float by, float bz, float cx, float cy,
@@ -403,6 +318,11 @@ template <typename T>
 __device__ __forceinline__ bool strictly_inside(const Dev<T>& d, T px, T py, T pz, int4 t) {
   return strictly_inside_at(d.X, px, py, pz, t);
 }
+// The same behind a call: where it is rare, its registers stay out of the caller.
+template <typename T>
+__device__ __noinline__ bool strictly_inside_call(const R4<T>* X, T px, T py, T pz, int4 t) {
+  return strictly_inside_at(X, px, py, pz, t);
+}
 
 // Obstacle tests of one query point (Eq. 4): the sphere whose signed surface
 // distance |x - c_j| - r_j is smallest among those strictly containing it
@@ -448,16 +368,13 @@ __device__ __forceinline__ void obstacle_tests(const Dev<T>& d, T px, T py, T pz
   }
   if (d.ot.n > 0)
     bvh_point_query(d.ot, 0, (double)px, (double)py, (double)pz, [&](int e) {
-      if (strictly_inside_at(d.OX, px, py, pz, d.ot.prim[e])) ++n_mesh;
+      if (strictly_inside_call(d.OX, px, py, pz, d.ot.prim[e])) ++n_mesh;
     });
 }
 
 template <typename T>
 __device__ void spring_update_vertex(const Dev<T>& d, int qi, int& active_out, unsigned long long& ssig);
 
-// One warp per query vertex: the lanes test the candidates of the vertex's
-// hash bucket in parallel; hits are merged by lane 0 into the vertex's sorted,
-// duplicate-free pair list.
 // Block totals of one narrow-phase-and-spring-update launch into this
 // iteration's record: self pairs, obstacle pairs, finished springs and the
 // springs' signature.
@@ -476,84 +393,300 @@ __device__ __forceinline__ void narrow_block_totals(const Dev<T>& d, int n_self,
   }
 }
 
-template <typename T, int BS>
-__global__ void __launch_bounds__(BS) k_narrow(Dev<T> d) {
+// l1 norm, and triple product a . (b x c), in FP32.
+__device__ __forceinline__ float l1(const float (&a)[3]) { return fabsf(a[0]) + fabsf(a[1]) + fabsf(a[2]); }
+__device__ __forceinline__ float triple(const float (&a)[3], const float (&b)[3], const float (&c)[3]) {
+  return a[0] * (b[1] * c[2] - b[2] * c[1]) + a[1] * (b[2] * c[0] - b[0] * c[2]) + a[2] * (b[0] * c[1] - b[1] * c[0]);
+}
+
+static constexpr int BRICK = 3;  // edge of the bricks of cells that k_tets looks up at once
+
+// Empty slot of a pair list (above every tet id).
+static constexpr int NO_PAIR = 0x7FFFFFFF;
+
+// Enters query vertex qi at position p (internal vertex v, robot rv) into the
+// list of its cell, and clears its pair list.
+template <typename T>
+__device__ __forceinline__ void bin_query(const Dev<T>& d, int qi, int v, int rv, R4<T> p) {
+  d.pair_count[qi] = 0;
+  int* out = d.pair_tet + (size_t)qi * d.max_pairs;
+  for (int k = 0; k < d.max_pairs; ++k) out[k] = NO_PAIR;
+  if (!(d.collision >= 1 && isfinite(p.x) && isfinite(p.y) && isfinite(p.z))) return;
+  const float inv = (float)d.inv_cell, x = (float)p.x, y = (float)p.y, z = (float)p.z;
+  const int cx = cell_coord_f(x, inv), cy = cell_coord_f(y, inv), cz = cell_coord_f(z, inv);
+  d.q_pos[qi] = make_float4(x, y, z, __int_as_float(v));
+  d.q_next[qi] = atomicExch(&d.q_head[hash_cell(cx, cy, cz, rv) & (d.H_q - 1u)], qi + 1);
+  // (a word's 32 cells overlap the next word's first 16, see k_tets; only the
+  // first BRICK - 1 of those are looked up there)
+  const unsigned words = d.H_q / 8 - 1u;
+  atomicOr(&d.q_bits[hash_cell(cx >> 4, cy, cz, rv) & words], 1u << (cx & 15));
+  if ((cx & 15) < BRICK - 1) atomicOr(&d.q_bits[hash_cell((cx >> 4) - 1, cy, cz, rv) & words], 0x10000u << (cx & 15));
+}
+
+static constexpr int QUERY_THREADS = 128;
+
+// One thread per query vertex: its cell's list, and its obstacle tests.
+template <typename T>
+__global__ void __launch_bounds__(QUERY_THREADS, 4) k_queries(Dev<T> d) {
   __shared__ int shi[32];
-  const int lane = threadIdx.x & 31;
-  const int qi = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
-  int n_self = 0, n_obs = 0, n_spr = 0;
-  unsigned long long ssig = 0;
+  const int qi = blockIdx.x * QUERY_THREADS + threadIdx.x;
+  int n_obs = 0;
   if (qi < d.n_q) {
     const int v = d.q_verts[qi];
-    const R4<T> pv = d.X[v];
-    const T px = pv.x, py = pv.y, pz = pv.z;
-    int cnt = 0;
-    bool over = false;
-    int* out = d.pair_tet + (size_t)qi * d.max_pairs;
-    const int rv = d.robot_of_vert ? d.robot_of_vert[v] : 0;
-    if (d.collision >= 1 && isfinite(px) && isfinite(py) && isfinite(pz)) {
-      int cp[3];
-      if constexpr (std::is_same<T, float>::value) {
-        const float inv_f = (float)d.inv_cell;
-        cp[0] = cell_coord_f(px, inv_f);
-        cp[1] = cell_coord_f(py, inv_f);
-        cp[2] = cell_coord_f(pz, inv_f);
-      } else {
-        cp[0] = cell_coord((double)px, d.inv_cell);
-        cp[1] = cell_coord((double)py, d.inv_cell);
-        cp[2] = cell_coord((double)pz, d.inv_cell);
-      }
-      const unsigned h = hash_cell(cp[0], cp[1], cp[2], rv) & (d.H_t - 1u);
-      const int b0 = d.cell_start[h];
-      const int b1 = min(d.cell_start[h + 1], d.cap_items);
-      for (int base = b0; base < b1; base += 32) {
-        const int k = base + lane;
-        int e = -1;
-        bool hit = false;
-        if (k < b1) {
-          e = chk_idx(d.ctrl, d.items[k], d.n_t);
-          const int4 t = chk_idx4(d.ctrl, d.tet[e], d.n_v);
-          const bool same_robot = !d.robot_of_tet || d.robot_of_tet[e] == rv;
-          if (same_robot && t.x != v && t.y != v && t.z != v && t.w != v) hit = strictly_inside(d, px, py, pz, t);
+    const R4<T> p = d.X[v];
+    bin_query(d, qi, v, d.robot_of_vert ? d.robot_of_vert[v] : 0, p);
+    int best, n_sph, n_mesh;
+    obstacle_tests(d, p.x, p.y, p.z, best, n_sph, n_mesh);
+    n_obs = n_sph + n_mesh;
+    d.obs_sphere[qi] = best;
+    if (d.obs_mesh) d.obs_mesh[qi] = n_mesh;
+  }
+  if (d.collision < 2) return;
+  const int s = block_sum_int(n_obs, shi);
+  if (threadIdx.x == 0 && s) atomicAdd(&(d.hist + (d.ctrl->iter % d.hist_cap))->n_obstacle_pairs, s);
+}
+
+// FP32 test of a point against a tet, corners given as differences from the
+// point: false only if one of the four orientation signs of the exact test is
+// certainly negative.  Each sign is a triple product of differences, whose FP32
+// rounding error is below 8 u times the product of the factors' 1-norms
+// (u = 2^-24; 1e-6 = 16.8 u is used); dl bounds the error that rounded FP64
+// positions add to a difference.  The constant covers underflow; differences
+// above 1e9 (products that could overflow) and NaN pass, like every value
+// within its bound.
+__device__ __forceinline__ bool may_be_inside(const float (&a)[3], const float (&b)[3], const float (&c)[3],
+                                              const float (&e)[3], float dl) {
+  const float na = l1(a) + dl, nb = l1(b) + dl, nc = l1(c) + dl, ne = l1(e) + dl;
+  if (!(na + nb + nc + ne < 1e9f)) return true;
+  const float tiny = 1e-25f, k = 1e-6f;
+  const float ab = na * nb, ce = nc * ne;
+  const float e0 = k * nb * ce + dl * (nb * nc + ce + nb * ne) + tiny, e1 = k * na * ce + dl * (na * nc + ce + na * ne) + tiny,
+              e2 = k * ab * ne + dl * (ab + na * ne + nb * ne) + tiny, e3 = k * ab * nc + dl * (ab + na * nc + nb * nc) + tiny;
+  return !(triple(b, c, e) < -e0 || triple(a, c, e) > e1 || triple(a, b, e) < -e2 || triple(a, b, c) > e3);
+}
+
+// Enters tet e into the pair list of query vertex qi: slot k keeps the smallest
+// id it is given and passes the other on, so the list ends as the smallest
+// max_pairs ids in ascending order whatever the order of arrival.
+template <typename T>
+__device__ __forceinline__ void add_pair(const Dev<T>& d, int qi, int e) {
+  if (atomicAdd(&d.pair_count[qi], 1) >= d.max_pairs) set_status(d.ctrl, ST_PAIRS_TRUNC);
+  int* out = d.pair_tet + (size_t)qi * d.max_pairs;
+  for (int k = 0; k < d.max_pairs; ++k) {
+    const int old = atomicMin(&out[k], e);
+    if (old == NO_PAIR) break;
+    e = max(old, e);
+  }
+}
+
+__device__ __forceinline__ bool finite_t(float x) { return isfinite(x); }
+__device__ __forceinline__ bool finite_t(double x) { return (__double2hiint(x) & 0x7FF00000) != 0x7FF00000; }
+
+// Narrow phase, one thread per tet, over the cells of the tet's box: tests the
+// query vertices listed in them whose own cell is the visited one (so every
+// vertex of the box is met once).
+//
+// The lists hold the boundary vertices alone, far fewer entries than a hash of
+// the tets needs.  Most cells are empty; a table of one bit per cell, small
+// enough for the first-level cache, shows which, for a brick of 3 x 3 x 3 cells
+// with nine independent reads (a word holds 32 cells along x, starting every 16,
+// so that three neighbours always share one).  What is left is uneven, so each
+// warp works it off together: its lanes append (tet, cell, first vertex) for the
+// occupied cells to a queue, then each takes one entry, tests its vertex in FP32
+// (own cell, box, signs) and appends the next one of the list.  The vertices that
+// pass go to a second queue, and the exact tests, which may need FP64 or longer
+// arithmetic, run on 32 of them at a time.
+// CHECK: the tets are a caller's and their vertex ids are tested first.
+// Measured (k_tets with k_queries, the faces' hash beside them) against a hash of
+// all tets (count, scan, fill) and one warp per vertex: 117 and 321 us for
+// 983,040 tets, 37 and 98 us for 193,920, 42 and 140 us for 51,840 in FP64.  Two
+// to five blocks of 256 threads to an SM measured alike; blocks of 64 or 128
+// threads, which each need the same shared memory, are slower at large sizes.
+static constexpr int TETS_MAX_THREADS = 256;
+
+template <typename T, bool CHECK>
+__global__ void __launch_bounds__(TETS_MAX_THREADS, 4) k_tets(Dev<T> d) {
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr int WARPS = TETS_MAX_THREADS / 32;
+  __shared__ unsigned s_entries;
+  __shared__ int4 s_visits[WARPS][64], s_tet[WARPS][32];  // (cell, 32 x list entry + lane); vertex ids
+  __shared__ int2 s_pairs[WARPS][64];                     // (tet, query vertex)
+  __shared__ float s_x[WARPS][12][32];                    // corners
+  if (threadIdx.x == 0) s_entries = 0;
+  __syncthreads();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const unsigned before = (1u << lane) - 1u;
+  int c0[3] = {0, 0, 0}, n[3] = {1, 1, 1}, ncell = 0;
+  const float inv = (float)d.inv_cell;
+  if (i < d.n_t) {
+    int4 t = d.tet[i];
+    bool valid = true;
+    if (CHECK) {
+      const unsigned nv = (unsigned)d.n_v;
+      valid = (unsigned)t.x < nv && (unsigned)t.y < nv && (unsigned)t.z < nv && (unsigned)t.w < nv;
+      if (!valid) set_status(d.ctrl, ST_BAD_INPUT);
+    } else {
+      t = chk_idx4(d.ctrl, t, d.n_v);
+    }
+    if (valid) {
+      const R4<T> p[4] = {d.X[t.x], d.X[t.y], d.X[t.z], d.X[t.w]};
+      // (rounding is monotone: the rounded box holds the rounded image of every
+      // point of the tet, and so do the cells of its corners)
+      float lo[3], hi[3];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        valid = valid && finite_t(p[k].x) && finite_t(p[k].y) && finite_t(p[k].z);
+        const float x[3] = {(float)p[k].x, (float)p[k].y, (float)p[k].z};
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          s_x[wid][3 * k + j][lane] = x[j];
+          lo[j] = k ? fminf(lo[j], x[j]) : x[j];
+          hi[j] = k ? fmaxf(hi[j], x[j]) : x[j];
         }
-        unsigned m = __ballot_sync(0xffffffffu, hit);
-        while (m) {
-          const int src = __ffs(m) - 1;
-          m &= m - 1;
-          const int eh = __shfl_sync(0xffffffffu, e, src);
-          if (lane == 0) {
-            // sorted insert without duplicates (a tet may repeat in a bucket)
-            int pos = 0;
-            while (pos < cnt && out[pos] < eh) ++pos;
-            if (!(pos < cnt && out[pos] == eh)) {
-              bool ins = true;
-              if (cnt == d.max_pairs) {
-                over = true;
-                if (pos == cnt) ins = false;
-                else --cnt;  // drop the largest to keep the smallest ids
-              }
-              if (ins) {
-                for (int j = cnt; j > pos; --j) out[j] = out[j - 1];
-                out[pos] = eh;
-                ++cnt;
-              }
-            }
+      }
+      if (!valid) {
+        set_status(d.ctrl, ST_NONFINITE);
+      } else {
+        s_tet[wid][lane] = t;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          c0[j] = cell_coord_f(lo[j], inv);
+          n[j] = cell_coord_f(hi[j], inv) - c0[j] + 1;
+        }
+        const long long m = (long long)n[0] * n[1] * n[2];
+        if (m > MAX_CELLS_PER_ITEM) set_status(d.ctrl, ST_OVERFLOW);
+        else ncell = (int)m;
+      }
+    }
+  }
+  {
+    const unsigned m = __reduce_add_sync(FULL, (unsigned)ncell);
+    if (lane == 0 && m) atomicAdd(&s_entries, m);
+    __syncthreads();
+    if (threadIdx.x == 0) add_entries(d, (unsigned long long)s_entries);
+  }
+  const int rt = d.robot_of_tet && i < d.n_t ? d.robot_of_tet[i] : 0;
+  int bx = 0, by = 0, bz = ncell > 0 ? 0 : n[2];  // this lane's next brick (relative to the box),
+  int ox = 0, oy = 0, oz = 0;                     //   the one before it,
+  unsigned occ = 0;                               //   and that one's occupied cells not yet queued
+  int n_visits = 0, n_pairs = 0;  // queued (the same in all lanes)
+  for (;;) {
+    while (n_visits < 32) {
+      if (!__any_sync(FULL, occ || bz < n[2])) break;
+      if (!occ && bz < n[2]) {
+        const int cx = c0[0] + bx, shift = cx & 15;
+        const unsigned keep = (1u << min(BRICK, n[0] - bx)) - 1u;
+        unsigned row[BRICK * BRICK];
+#pragma unroll
+        for (int r = 0; r < BRICK * BRICK; ++r) {
+          const int y = by + r % BRICK, z = bz + r / BRICK;
+          row[r] = y < n[1] && z < n[2]
+                       ? __ldg(&d.q_bits[hash_cell(cx >> 4, c0[1] + y, c0[2] + z, rt) & (d.H_q / 8 - 1u)])
+                       : 0u;
+        }
+#pragma unroll
+        for (int r = 0; r < BRICK * BRICK; ++r) occ |= (row[r] >> shift & keep) << (BRICK * r);
+        ox = bx, oy = by, oz = bz;
+        if ((bx += BRICK) >= n[0]) {
+          bx = 0;
+          if ((by += BRICK) >= n[1]) {
+            by = 0;
+            bz += BRICK;
           }
         }
       }
+      int head = 0;
+      int4 visit = make_int4(0, 0, 0, 0);
+      if (occ) {
+        const int b = __ffs(occ) - 1;
+        occ &= occ - 1;
+        visit = make_int4(c0[0] + ox + b % BRICK, c0[1] + oy + b / BRICK % BRICK, c0[2] + oz + b / (BRICK * BRICK), 0);
+        head = __ldg(&d.q_head[hash_cell(visit.x, visit.y, visit.z, rt) & (d.H_q - 1u)]);
+      }
+      const unsigned who = __ballot_sync(FULL, head);
+      visit.w = head * 32 + lane;
+      if (head) s_visits[wid][n_visits + __popc(who & before)] = visit;
+      n_visits += __popc(who);
     }
-    if (lane == 0) {
-      if (over) set_status(d.ctrl, ST_PAIRS_TRUNC);
-      d.pair_count[qi] = cnt;
-      n_self = cnt;
-      int best, n_sph, n_mesh;
-      obstacle_tests(d, px, py, pz, best, n_sph, n_mesh);
-      n_obs = n_sph + n_mesh;
-      d.obs_sphere[qi] = best;
-      if (d.obs_mesh) d.obs_mesh[qi] = n_mesh;
+    __syncwarp();
+    // one vertex to each lane
+    const int take = min(n_visits, 32);
+    const bool mine = lane < take;
+    int4 visit = make_int4(0, 0, 0, 0);
+    if (mine) visit = s_visits[wid][n_visits - 1 - lane];
+    __syncwarp();
+    n_visits -= take;
+    bool cand = false;
+    int qi = 0, next = 0;
+    const int src = visit.w & 31;
+    if (mine) {
+      qi = chk_idx(d.ctrl, (int)((unsigned)visit.w >> 5) - 1, d.n_q);
+      const float4 p = __ldg(&d.q_pos[qi]);
+      next = __ldg(&d.q_next[qi]);
+      const int v = __float_as_int(p.w);
+      const int4 t = s_tet[wid][src];
+      if (cell_coord_f(p.x, inv) == visit.x && cell_coord_f(p.y, inv) == visit.y && cell_coord_f(p.z, inv) == visit.z &&
+          t.x != v && t.y != v && t.z != v && t.w != v) {
+        // corners relative to the vertex (a difference of floats has its exact
+        // sign, so the closed box test is exact; the exact test has the open one)
+        float e[4][3], dl = 0.0f;
+        const float pp[3] = {p.x, p.y, p.z};
+        bool in_box = true;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float x = s_x[wid][3 * k + j][src];
+            e[k][j] = x - pp[j];
+            if constexpr (!std::is_same<T, float>::value) dl += fabsf(x);
+          }
+          if constexpr (!std::is_same<T, float>::value) dl += fabsf(pp[j]);
+          in_box = in_box && min4(e[0][j], e[1][j], e[2][j], e[3][j]) <= 0.0f && max4(e[0][j], e[1][j], e[2][j], e[3][j]) >= 0.0f;
+        }
+        cand = in_box && may_be_inside(e[0], e[1], e[2], e[3], 0x1p-22f * dl);
+      }
+    }
+    const unsigned again = __ballot_sync(FULL, next), who = __ballot_sync(FULL, cand);
+    visit.w = next * 32 + src;
+    if (next) s_visits[wid][n_visits + __popc(again & before)] = visit;
+    n_visits += __popc(again);
+    if (cand) s_pairs[wid][n_pairs + __popc(who & before)] = make_int2(i - lane + src, qi);
+    n_pairs += __popc(who);
+    const bool last = take == 0;
+    if (n_pairs >= 32 || last) {
+      __syncwarp();
+      const int m = min(n_pairs, 32);
+      if (lane < m) {
+        const int2 pr = s_pairs[wid][n_pairs - 1 - lane];
+        const int v = d.q_verts[pr.y];
+        if (!d.robot_of_tet || d.robot_of_vert[v] == d.robot_of_tet[pr.x]) {
+          // (strictly_inside, with the four signs in a loop around one inlined
+          // copy of the exact arithmetic: a call would cost the walk its registers)
+          const R4<T> x = d.X[v];
+          const int4 pt = d.tet[pr.x];
+          const R4<T> p[4] = {d.X[pt.x], d.X[pt.y], d.X[pt.z], d.X[pt.w]};
+          bool in = x.x > min4(p[0].x, p[1].x, p[2].x, p[3].x) && x.x < max4(p[0].x, p[1].x, p[2].x, p[3].x) &&
+                    x.y > min4(p[0].y, p[1].y, p[2].y, p[3].y) && x.y < max4(p[0].y, p[1].y, p[2].y, p[3].y) &&
+                    x.z > min4(p[0].z, p[1].z, p[2].z, p[3].z) && x.z < max4(p[0].z, p[1].z, p[2].z, p[3].z);
+#pragma unroll 1
+          for (int s = 0; s < 4 && in; ++s) {
+            const R4<T> a = s == 0 ? x : p[0], b = s == 1 ? x : p[1], e = s == 2 ? x : p[2], f = s == 3 ? x : p[3];
+            int sign = 0;
+            if constexpr (std::is_same<T, float>::value)
+              sign = orient_filter_f(a.x, a.y, a.z, b.x, b.y, b.z, e.x, e.y, e.z, f.x, f.y, f.z);
+            if (sign == 0) sign = orient_filter(a.x, a.y, a.z, b.x, b.y, b.z, e.x, e.y, e.z, f.x, f.y, f.z);
+            if (sign == 0) sign = orient_exact_inline(a.x, a.y, a.z, b.x, b.y, b.z, e.x, e.y, e.z, f.x, f.y, f.z);
+            in = sign > 0;
+          }
+          if (in) add_pair(d, pr.y, pr.x);
+        }
+      }
+      __syncwarp();
+      n_pairs -= m;
+      if (last && n_pairs == 0) break;
     }
   }
-  narrow_block_totals(d, n_self, n_obs, n_spr, ssig, shi);
 }
 
 // ---- AABB trees: refit and point queries ----
@@ -820,9 +953,9 @@ __device__ int closest_face_warp(const Dev<T>& d, int v, int rv, V3 o, double& r
     for (int idx = lane; idx < ncell; idx += 32) {
       const int dx = idx % side - k, dy = (idx / side) % side - k, dz = idx / (side * side) - k;
       if (max(abs(dx), max(abs(dy), abs(dz))) != k) continue;
-      const unsigned h = d.H_t + (hash_cell(c0[0] + dx, c0[1] + dy, c0[2] + dz, rv) & (d.H_f - 1u));
-      const int k0 = d.cell_start[h], k1 = min(d.cell_start[h + 1], d.cap_items);
-      for (int q = k0; q < k1; ++q) closest_candidate(d, v, rv, d.items[q] - d.n_t, o, lf, ld, l1, l2);
+      const int2 r = d.cell_range[hash_cell(c0[0] + dx, c0[1] + dy, c0[2] + dz, rv) & (d.H_f - 1u)];
+      const int k1 = min(r.y, d.cap_items);
+      for (int q = r.x; q < k1; ++q) closest_candidate(d, v, rv, d.items[q], o, lf, ld, l1, l2);
     }
     warp_argmin(lf, ld, l1, l2);
     if (lf >= 0 && (best_f < 0 || ld < bestd || (ld == bestd && lf < best_f))) {
@@ -1057,10 +1190,14 @@ template <typename T>
 __global__ void __launch_bounds__(128) k_springs(Dev<T> d) {
   __shared__ int shi[32];
   const int qi = blockIdx.x * blockDim.x + threadIdx.x;
-  int n_spr = 0;
+  int n_self = 0, n_spr = 0;
   unsigned long long ssig = 0;
-  if (qi < d.n_q) spring_update_vertex(d, qi, n_spr, ssig);
-  narrow_block_totals(d, 0, 0, n_spr, ssig, shi);
+  if (qi < d.n_q) {
+    n_self = d.pair_count[qi];
+    if (n_self > d.max_pairs) d.pair_count[qi] = n_self = d.max_pairs;
+    spring_update_vertex(d, qi, n_spr, ssig);
+  }
+  narrow_block_totals(d, n_self, 0, n_spr, ssig, shi);
 }
 
 // FP32 test of a face against a ray from o along the unit direction dir, which
@@ -1073,10 +1210,6 @@ __global__ void __launch_bounds__(128) k_springs(Dev<T> d) {
 // rounded to FP32, which adds dl = 2^-22 times the coordinates' sizes to every
 // difference.  The constant covers underflow, differences above 1e9 (products
 // that could overflow) and NaN pass, like every value within its bound.
-__device__ __forceinline__ float l1(const float (&a)[3]) { return fabsf(a[0]) + fabsf(a[1]) + fabsf(a[2]); }
-__device__ __forceinline__ float triple(const float (&a)[3], const float (&b)[3], const float (&c)[3]) {
-  return a[0] * (b[1] * c[2] - b[2] * c[1]) + a[1] * (b[2] * c[0] - b[0] * c[2]) + a[2] * (b[0] * c[1] - b[1] * c[0]);
-}
 template <typename T>
 __device__ __forceinline__ bool face_may_hit(const R4<T>& q0, const R4<T>& q1, const R4<T>& q2, const float (&o)[3],
                                              const float (&dir)[3]) {
@@ -1199,9 +1332,9 @@ __global__ void __launch_bounds__(CAST_THREADS) k_cast(Dev<T> d) {
     bool walking = valid;             // team-uniform, like the walk's whole state
     int steps = 0, kk = 0, k1 = 0;    // cells left behind; the next entry of this cell and its end
     auto enter = [&]() {
-      const unsigned h = d.H_t + (hash_cell(cell[0], cell[1], cell[2], rv) & (d.H_f - 1u));
-      kk = d.cell_start[h];
-      k1 = min(d.cell_start[h + 1], d.cap_items);
+      const int2 r = d.cell_range[hash_cell(cell[0], cell[1], cell[2], rv) & (d.H_f - 1u)];
+      kk = r.x;
+      k1 = min(r.y, d.cap_items);
     };
     if (walking) enter();
     while (__any_sync(FULL, walking)) {
@@ -1211,7 +1344,7 @@ __global__ void __launch_bounds__(CAST_THREADS) k_cast(Dev<T> d) {
         if (kk < k1) {
           const int k = kk + tl;
           if (k < k1) {
-            const int f = d.items[k] - d.n_t;
+            const int f = d.items[k];
             if (!d.robot_of_face || d.robot_of_face[f] == rv) {
               const int4 fv = chk_face(d.ctrl, d.faces[chk_idx(d.ctrl, f, d.n_f)], d.n_v);
               if (fv.x != v && fv.y != v && fv.z != v && face_may_hit(d.X[fv.x], d.X[fv.y], d.X[fv.z], of, df)) cand = f;
@@ -1404,59 +1537,81 @@ void launch_bvh_refit(const BvhDev& b, const R4<T>* X, cudaStream_t st) {
   k_bvh_refit<T><<<(b.n + 255) / 256, 256, 0, st>>>(b, X);
 }
 
+// First of the broad phase; both sides below follow it.
 template <typename T>
-void launch_collision(const Dev<T>& d, const CollisionScratch& cs, cudaStream_t st) {
+void launch_broad_clear(const Dev<T>& d, const CollisionScratch& cs, cudaStream_t st) {
+  if (d.broad != 1) cudaMemsetAsync(cs.zero, 0, cs.zero_bytes, st);
+}
+
+// Face side, read by the ray casts alone.
+template <typename T>
+void launch_faces(const Dev<T>& d, cudaStream_t st) {
   if (d.broad == 1) {
-    // AABB trees: refit the tet and face trees to this iteration's positions
-    launch_bvh_refit<T>(d.bt, d.X, st);
     launch_bvh_refit<T>(d.bf, d.X, st);
+    return;
+  }
+  if (d.n_f <= 0) return;
+  const int nb = (d.n_f + FACE_THREADS - 1) / FACE_THREADS;
+  k_faces<T, false><<<nb, FACE_THREADS, 0, st>>>(d);
+  k_place_cells<T><<<((int)d.H_f + SCAN_TILE - 1) / SCAN_TILE, SCAN_THREADS, 0, st>>>(d);
+  k_faces<T, true><<<nb, FACE_THREADS, 0, st>>>(d);
+}
+
+// Narrow phase over the tets once the query vertices are in their lists.
+template <typename T>
+void launch_tets(const Dev<T>& d, bool check, cudaStream_t st) {
+  const int bs = d.narrow_threads > 0 ? std::min(d.narrow_threads, TETS_MAX_THREADS) : TETS_MAX_THREADS, nb = (d.n_t + bs - 1) / bs;
+  if (check)
+    k_tets<T, true><<<nb, bs, 0, st>>>(d);
+  else
+    k_tets<T, false><<<nb, bs, 0, st>>>(d);
+}
+
+// A caller's positions into the kernels' layout, and its query vertices, whose
+// ids are tested first, into their lists.
+__global__ void __launch_bounds__(QUERY_THREADS) k_pack_queries(Dev<float> d, const float* __restrict__ xyz,
+                                                                R4<float>* __restrict__ X) {
+  const int i = blockIdx.x * QUERY_THREADS + threadIdx.x;
+  if (i < d.n_v) X[i] = R4<float>{xyz[3 * i], xyz[3 * i + 1], xyz[3 * i + 2], 0.0f};
+  if (i < d.n_q) {
+    const int v = d.q_verts[i];
+    if (v < 0 || v >= d.n_v) set_status(d.ctrl, ST_BAD_INPUT);
+    else bin_query(d, i, v, 0, R4<float>{xyz[3 * v], xyz[3 * v + 1], xyz[3 * v + 2], 0.0f});
+  }
+}
+
+void launch_pack_queries(const Dev<float>& d, const float* xyz, R4<float>* X, cudaStream_t st) {
+  k_pack_queries<<<(std::max(d.n_v, d.n_q) + QUERY_THREADS - 1) / QUERY_THREADS, QUERY_THREADS, 0, st>>>(d, xyz, X);
+}
+
+// Pairs and obstacle contacts.
+template <typename T>
+void launch_collision(const Dev<T>& d, cudaStream_t st) {
+  if (d.broad == 1) {
+    // AABB tree: refit the tet tree to this iteration's positions
+    launch_bvh_refit<T>(d.bt, d.X, st);
     if (d.n_q > 0)
       k_narrow_bvh<T><<<(d.n_q + NARROW_BVH_THREADS - 1) / NARROW_BVH_THREADS, NARROW_BVH_THREADS, 0, st>>>(d);
     return;
   }
-  const int n_items = d.n_t + d.n_f;
-  const int H = (int)(d.H_t + d.H_f);
-  // with the single-pass scan its status words and ticket follow the counts
-  // and are zeroed by the same memset
-  const size_t n_zero = (size_t)(H + 1) + (cs.tile_status ? (size_t)scan_lookback_extra_ints(H + 1) : 0);
-  cudaMemsetAsync(d.cell_count, 0, sizeof(int) * n_zero, st);
-  cudaMemsetAsync(d.cell_cursor, 0, sizeof(int) * (size_t)H, st);
-  k_grid_bin<T, false><<<(n_items + 255) / 256, 256, 0, st>>>(d);
-  const int n_scan = H + 1;
-  const int n_tiles = (n_scan + SCAN_TILE - 1) / SCAN_TILE;
-  if (cs.tile_status) {
-    k_scan_lookback<<<n_tiles, SCAN_THREADS, 0, st>>>(d.cell_count, d.cell_start, n_scan, cs.tile_status, cs.ticket,
-                                                       cs.total, d.ctrl, d.cap_items, d.wait_budget);
-  } else {
-    k_scan_tiles<<<n_tiles, SCAN_THREADS, 0, st>>>(d.cell_count, d.cell_start, cs.tile_sums, n_scan);
-    k_scan_top<<<1, 1024, 0, st>>>(cs.tile_sums, n_tiles, cs.total, d.ctrl, d.cap_items);
-    k_scan_add<<<(n_scan + 255) / 256, 256, 0, st>>>(d.cell_start, cs.tile_sums, n_scan);
-  }
-  k_grid_bin<T, true><<<(n_items + 255) / 256, 256, 0, st>>>(d);
-  if (d.n_q > 0) {
-    const long long threads = 32LL * d.n_q;
-    const int bs = d.narrow_threads > 0 ? d.narrow_threads : 256;
-    const unsigned nb = (unsigned)((threads + bs - 1) / bs);
-    if (bs == 128)
-      k_narrow<T, 128><<<nb, 128, 0, st>>>(d);
-    else if (bs == 512)
-      k_narrow<T, 512><<<nb, 512, 0, st>>>(d);
-    else
-      k_narrow<T, 256><<<nb, 256, 0, st>>>(d);
-  }
+  k_queries<T><<<(d.n_q + QUERY_THREADS - 1) / QUERY_THREADS, QUERY_THREADS, 0, st>>>(d);
+  launch_tets<T>(d, false, st);
 }
 
 // The spring update (a separate launch after the hash's narrow phase, inside
 // the tree's narrow phase), then the ray casts of the vertices it queued.
+// These wait for faces_ready (unless null): the face side may be on a branch of
+// its own.
 template <typename T>
-void launch_springs(const Dev<T>& d, cudaStream_t st) {
+void launch_springs(const Dev<T>& d, cudaStream_t st, cudaEvent_t faces_ready) {
   if (d.n_q <= 0) return;
   if (d.broad != 1) k_springs<T><<<(d.n_q + 127) / 128, 128, 0, st>>>(d);
-  // enough teams for one pass over a list of up to 32,768 casts
+  if (faces_ready) cudaStreamWaitEvent(st, faces_ready, 0);
   if (d.broad == 1) {
     k_cast_bvh<T><<<std::min((d.n_q + CAST_THREADS - 1) / CAST_THREADS, 1024), CAST_THREADS, 0, st>>>(d);
     return;
   }
+  // enough teams for one pass over a list of up to 32,768 casts
   const int per_block = CAST_THREADS / 8;
   const int blocks = std::min((d.n_q + per_block - 1) / per_block, 1024);
   k_cast<T><<<blocks, CAST_THREADS, 0, st>>>(d);
@@ -1467,15 +1622,20 @@ void launch_scan_exclusive(const int* in, int* out, int n, int* tile_sums, int* 
   if (n <= 0) return;
   const int n_tiles = scan_tiles(n);
   k_scan_tiles<<<n_tiles, SCAN_THREADS, 0, st>>>(in, out, tile_sums, n);
-  k_scan_top<<<1, 1024, 0, st>>>(tile_sums, n_tiles, total, nullptr, 0);
+  k_scan_top<<<1, 1024, 0, st>>>(tile_sums, n_tiles, total);
   k_scan_add<<<(n + 255) / 256, 256, 0, st>>>(out, tile_sums, n);
 }
 
 template void launch_bvh_refit<float>(const BvhDev&, const R4<float>*, cudaStream_t);
 template void launch_bvh_refit<double>(const BvhDev&, const R4<double>*, cudaStream_t);
-template void launch_collision<float>(const Dev<float>&, const CollisionScratch&, cudaStream_t);
-template void launch_collision<double>(const Dev<double>&, const CollisionScratch&, cudaStream_t);
-template void launch_springs<float>(const Dev<float>&, cudaStream_t);
-template void launch_springs<double>(const Dev<double>&, cudaStream_t);
+template void launch_broad_clear<float>(const Dev<float>&, const CollisionScratch&, cudaStream_t);
+template void launch_broad_clear<double>(const Dev<double>&, const CollisionScratch&, cudaStream_t);
+template void launch_collision<float>(const Dev<float>&, cudaStream_t);
+template void launch_collision<double>(const Dev<double>&, cudaStream_t);
+template void launch_tets<float>(const Dev<float>&, bool, cudaStream_t);
+template void launch_faces<float>(const Dev<float>&, cudaStream_t);
+template void launch_faces<double>(const Dev<double>&, cudaStream_t);
+template void launch_springs<float>(const Dev<float>&, cudaStream_t, cudaEvent_t);
+template void launch_springs<double>(const Dev<double>&, cudaStream_t, cudaEvent_t);
 
 }  // namespace casim

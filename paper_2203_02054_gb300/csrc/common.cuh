@@ -74,7 +74,6 @@ struct Ctrl {
   unsigned queue;        // next robot for the cluster PCG work queue
   long long iter;        // outer iterations completed (history index)
   long long total_pcg;   // PCG iterations summed over outer iterations
-  int n_items;           // spatial-hash entries of this iteration
   int n_cast;            // ray-cast list length of this iteration (reset at its end)
   long long box_lo[3];   // bounding box of all item boxes of this iteration,
   long long box_hi[3];   //   as order-preserving integer codes of doubles
@@ -188,12 +187,17 @@ struct Dev {
   const int4* faces;     // n_f (v0, v1, v2, owning tet)
   const double* spheres; // 4 n_spheres
   const float* spheres_f; // the same, rounded to FP32 (the reject test before the FP64 one)
-  unsigned H_t, H_f;     // hash sizes (powers of two)
-  int* cell_count;       // H_t + H_f (+1)
-  int* cell_start;       // H_t + H_f + 1
-  int* cell_cursor;      // H_t + H_f
-  int* items;            // cap_items
-  int cap_items;
+  unsigned H_q, H_f;     // hash sizes (powers of two): query vertices, boundary faces
+  int* q_head;           // H_q: 1 + first query vertex of the bucket's list, or 0
+  unsigned* q_bits;      // H_q / 8: the occupied cells, 32 along x to a word
+  int* q_next;           // n_q: the next entry of the vertex's list
+  float4* q_pos;         // n_q: its position in FP32 and its internal id (bits)
+  int* cell_count;       // H_f
+  int* cell_total;       // faces' entries
+  int2* cell_range;      // H_f: first and one past the last entry of the cell's faces in items
+  int* items;            // cap_items: face ids
+  int cap_items;         // entries that the faces and the tets may have together,
+  unsigned long long* entries; // and have
   int* pair_count;       // n_q
   int* pair_tet;         // n_q * max_pairs
   int* obs_sphere;       // n_q: sphere id or -1

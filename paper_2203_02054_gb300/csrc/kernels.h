@@ -7,14 +7,12 @@
 
 namespace casim {
 
+// What the hash broad phase zeroes each iteration (one piece): the number of
+// entries, the query vertices' list heads and bits, and the face cells' counts
+// with their total.
 struct CollisionScratch {
-  int* tile_sums;  // scan tiles of the hash count array
-  int* total;      // total hash entries
-  // single-pass scan (null: the three-kernel scan): per-tile status words and
-  // the tile ticket, stored right after the hash count array so that its one
-  // memset zeroes them too
-  unsigned long long* tile_status;
-  unsigned* ticket;
+  void* zero;
+  size_t zero_bytes;
 };
 
 static constexpr int LOCAL_THREADS = 128;
@@ -39,9 +37,16 @@ static constexpr size_t TEAM_SMEM_MAX = 216 * 1024;  //   dynamic shared memory
 static constexpr int PCG_CL_SIZE = 16;   // CTAs per cluster (non-portable size)
 
 template <typename T>
-void launch_collision(const Dev<T>& d, const CollisionScratch& cs, cudaStream_t st);
+void launch_broad_clear(const Dev<T>& d, const CollisionScratch& cs, cudaStream_t st);
 template <typename T>
-void launch_springs(const Dev<T>& d, cudaStream_t st);
+void launch_collision(const Dev<T>& d, cudaStream_t st);
+template <typename T>
+void launch_faces(const Dev<T>& d, cudaStream_t st);
+template <typename T>
+void launch_springs(const Dev<T>& d, cudaStream_t st, cudaEvent_t faces_ready);
+template <typename T>
+void launch_tets(const Dev<T>& d, bool check, cudaStream_t st);
+void launch_pack_queries(const Dev<float>& d, const float* xyz, R4<float>* X, cudaStream_t st);
 template <typename T>
 void launch_bvh_refit(const BvhDev& b, const R4<T>* X, cudaStream_t st);
 template <typename T>
@@ -155,6 +160,5 @@ int local_blocks(int n_t, int threads);
 int rhs_blocks(int n_free, int threads);
 int scan_tiles(int n);
 // ints to allocate after an (n + 1)-int count array for the single-pass scan
-int scan_lookback_extra_ints(int n);
 
 }  // namespace casim

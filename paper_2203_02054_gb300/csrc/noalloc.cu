@@ -2,7 +2,7 @@
 //
 // casim_contacts_noalloc runs the same spatial-hash broad phase and exact
 // narrow phase as a casim_step iteration, but keeps every intermediate buffer
-// (packed positions, hash counts and offsets, the hash entries, control words)
+// (packed positions, the query vertices' lists, the pair lists, control words)
 // in one file-scope device array instead of memory from cudaMalloc.  It exists
 // for callers that cannot allocate device memory while they run: real-time
 // controllers that must not allocate inside a control loop, and host programs
@@ -24,25 +24,26 @@ namespace {
 constexpr int NA_MAX_VERTS = 32768;
 constexpr int NA_MAX_TETS = 65536;
 constexpr int NA_MAX_QUERY = 16384;
-constexpr unsigned NA_HASH = 131072;  // power of two >= 2 * NA_MAX_TETS
+constexpr unsigned NA_HASH = 65536;  // power of two >= 4 * NA_MAX_QUERY
+constexpr int NA_MAX_PAIRS = 16;
 constexpr int NA_CAP_ITEMS = 16 * NA_MAX_TETS + 4096;
 
 // Byte offsets of the pieces inside the scratch array (each 256-byte aligned).
+// The first ones are zeroed by every call, as far as its hash needs.
 constexpr size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 constexpr size_t OFF_CTRL = 0;
-constexpr size_t OFF_HIST = align256(OFF_CTRL + sizeof(Ctrl));
-constexpr size_t OFF_X = align256(OFF_HIST + sizeof(IterRec));
-constexpr size_t OFF_COUNT = align256(OFF_X + sizeof(R4<float>) * NA_MAX_VERTS);
-constexpr size_t OFF_START = align256(OFF_COUNT + sizeof(int) * (NA_HASH + 2));
-constexpr size_t OFF_CURSOR = align256(OFF_START + sizeof(int) * (NA_HASH + 2));
-constexpr size_t OFF_ITEMS = align256(OFF_CURSOR + sizeof(int) * (NA_HASH + 1));
-constexpr size_t OFF_TILES = align256(OFF_ITEMS + sizeof(int) * NA_CAP_ITEMS);
-constexpr size_t OFF_TOTAL = align256(OFF_TILES + sizeof(int) * 1024);
-constexpr size_t OFF_OBS = align256(OFF_TOTAL + sizeof(int));
-constexpr size_t SCRATCH_BYTES = align256(OFF_OBS + sizeof(int) * NA_MAX_QUERY);
+constexpr size_t OFF_ENTRIES = align256(OFF_CTRL + sizeof(Ctrl));
+constexpr size_t OFF_BITS = align256(OFF_ENTRIES + sizeof(unsigned long long));
+constexpr size_t OFF_HEAD = align256(OFF_BITS + sizeof(unsigned) * (NA_HASH / 8));
+constexpr size_t OFF_X = align256(OFF_HEAD + sizeof(int) * NA_HASH);
+constexpr size_t OFF_NEXT = align256(OFF_X + sizeof(R4<float>) * NA_MAX_VERTS);
+constexpr size_t OFF_POS = align256(OFF_NEXT + sizeof(int) * NA_MAX_QUERY);
+constexpr size_t OFF_COUNT = align256(OFF_POS + sizeof(float4) * NA_MAX_QUERY);
+constexpr size_t OFF_PAIRS = align256(OFF_COUNT + sizeof(int) * NA_MAX_QUERY);
+constexpr size_t SCRATCH_BYTES = align256(OFF_PAIRS + sizeof(int) * NA_MAX_PAIRS * NA_MAX_QUERY);
 
-// The scratch: about 6.2 MiB, held by every GPU that loads the library until
-// the process exits.  Every call uses all of it, so calls whose GPU work
+// The scratch: about 2.2 MiB, held by every GPU that loads the library until
+// the process exits.  Every call uses it, so calls whose GPU work
 // overlaps (on different streams or host threads) race with each other.
 static __device__ __align__(256) unsigned char g_scratch[SCRATCH_BYTES];
 
@@ -54,32 +55,13 @@ static __device__ __align__(256) unsigned char g_scratch[SCRATCH_BYTES];
 std::mutex g_mu;
 void* g_addr[64] = {nullptr};
 
-// Control word and statistics record at the start of a call: zero, except the
-// bounding-box words, which start at the empty box (as a casim_step iteration
-// starts them) so that their atomic min / max reduce to the items' box.
-__global__ void k_init_ctrl(Ctrl* ctrl, IterRec* hist) {
-  if (threadIdx.x != 0) return;
-  Ctrl c{};
-  for (int j = 0; j < 3; ++j) {
-    c.box_lo[j] = 0x7FFFFFFFFFFFFFFFLL;
-    c.box_hi[j] = (long long)0x8000000000000000ULL;
-  }
-  *ctrl = c;
-  *hist = IterRec{};
-}
-
-__global__ void k_pack_and_check(const float* xyz, int n_verts, const int* tets, int n_tets, const int* query,
-                                 int n_query, R4<float>* X, Ctrl* ctrl) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n_verts) X[i] = R4<float>{xyz[3 * i], xyz[3 * i + 1], xyz[3 * i + 2], 0.0f};
-  if (i < 4 * n_tets) {
-    const int v = tets[i];
-    if (v < 0 || v >= n_verts) atomicOr(&ctrl->status, ST_BAD_INPUT);
-  }
-  if (i < n_query) {
-    const int v = query[i];
-    if (v < 0 || v >= n_verts) atomicOr(&ctrl->status, ST_BAD_INPUT);
-  }
+// The pair lists into the caller's arrays (a rejected call leaves them alone).
+__global__ void k_pairs_out(Dev<float> d, int* __restrict__ count, int* __restrict__ tets) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= d.n_q || (d.ctrl->status & ST_BAD_INPUT)) return;
+  const int n = min(d.pair_count[q], d.max_pairs);
+  count[q] = n;
+  for (int k = 0; k < n; ++k) tets[(size_t)q * d.max_pairs + k] = d.pair_tet[(size_t)q * d.max_pairs + k];
 }
 
 // Records the reason of a rejection for casim_last_error(NULL) on this thread.
@@ -125,55 +107,42 @@ extern "C" int casim_contacts_noalloc(int32_t n_verts, const float* dev_xyz, int
   unsigned char* base = static_cast<unsigned char*>(g_addr[dev]);
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   Ctrl* ctrl = reinterpret_cast<Ctrl*>(base + OFF_CTRL);
-  IterRec* hist = reinterpret_cast<IterRec*>(base + OFF_HIST);
   R4<float>* X = reinterpret_cast<R4<float>*>(base + OFF_X);
-  // the control word and the statistics record start from their initial values
-  k_init_ctrl<<<1, 32, 0, st>>>(ctrl, hist);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return fail(CASIM_E_CUDA, std::string("control init: ") + cudaGetErrorString(e));
-  int n_check = n_verts > 4 * n_tets ? n_verts : 4 * n_tets;
-  if (n_query > n_check) n_check = n_query;
-  k_pack_and_check<<<(n_check + 255) / 256, 256, 0, st>>>(dev_xyz, n_verts, dev_tets, n_tets, dev_query, n_query, X,
-                                                          ctrl);
-  int status = 0;
-  e = cudaMemcpyAsync(&status, &ctrl->status, sizeof(int), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) return fail(CASIM_E_CUDA, std::string("input check: ") + cudaGetErrorString(e));
-  if (status & ST_BAD_INPUT) return fail(CASIM_E_INVALID, "a tet or query vertex id is out of range");
-
   Dev<float> d{};
   d.n_v = n_verts;
   d.n_t = n_tets;
-  d.n_f = 0;
   d.n_q = n_query;
   d.X = X;
   d.tet = reinterpret_cast<const int4*>(dev_tets);
   d.q_verts = dev_query;
-  d.H_t = NA_HASH;
-  d.H_f = 1;
-  d.cell_count = reinterpret_cast<int*>(base + OFF_COUNT);
-  d.cell_start = reinterpret_cast<int*>(base + OFF_START);
-  d.cell_cursor = reinterpret_cast<int*>(base + OFF_CURSOR);
-  d.items = reinterpret_cast<int*>(base + OFF_ITEMS);
+  d.H_q = 64;
+  while (d.H_q < 4u * (unsigned)n_query) d.H_q *= 2;
+  d.q_bits = reinterpret_cast<unsigned*>(base + OFF_BITS);
+  d.q_head = reinterpret_cast<int*>(base + OFF_HEAD);
+  d.q_next = reinterpret_cast<int*>(base + OFF_NEXT);
+  d.q_pos = reinterpret_cast<float4*>(base + OFF_POS);
+  d.entries = reinterpret_cast<unsigned long long*>(base + OFF_ENTRIES);
   d.cap_items = NA_CAP_ITEMS;
-  d.pair_count = dev_pair_count;
-  d.pair_tet = dev_pair_tet;
-  d.obs_sphere = reinterpret_cast<int*>(base + OFF_OBS);
+  d.pair_count = reinterpret_cast<int*>(base + OFF_COUNT);
+  d.pair_tet = reinterpret_cast<int*>(base + OFF_PAIRS);
   d.max_pairs = max_pairs;
   d.collision = 1;
-  d.n_spheres = 0;
-  d.narrow_threads = 256;  // the regular narrow-phase launch shape; d.sp stays empty: no spring update
+  d.narrow_threads = 128;  // a few thousand tets: more, smaller blocks
   d.cell = cell_size;
   d.inv_cell = 1.0 / cell_size;
   d.ctrl = ctrl;
-  d.hist = hist;
-  d.hist_cap = 1;
-  CollisionScratch cs{reinterpret_cast<int*>(base + OFF_TILES), reinterpret_cast<int*>(base + OFF_TOTAL)};
-  launch_collision<float>(d, cs, st);
-  e = cudaGetLastError();
+  // zero control word, entries, bits and list heads; the vertex ids are tested
+  // where they are first used, so one wait at the end serves every check
+  cudaError_t e2 = cudaMemsetAsync(base, 0, OFF_HEAD + sizeof(int) * d.H_q, st);
+  launch_pack_queries(d, dev_xyz, X, st);
+  launch_tets<float>(d, true, st);
+  k_pairs_out<<<(n_query + 127) / 128, 128, 0, st>>>(d, dev_pair_count, dev_pair_tet);
+  e = e2 == cudaSuccess ? cudaGetLastError() : e2;
+  int status = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&status, &ctrl->status, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(CASIM_E_CUDA, std::string("contact check: ") + cudaGetErrorString(e));
+  if (status & ST_BAD_INPUT) return fail(CASIM_E_INVALID, "a tet or query vertex id is out of range");
   if (status & ST_NONFINITE) return fail(CASIM_E_NONFINITE, "non-finite position");
   if (status & ST_PAIRS_TRUNC)
     return fail(CASIM_E_OVERFLOW, "a query vertex lies in more than max_pairs tets (the smallest ids are kept)");

@@ -59,9 +59,9 @@ __device__ __forceinline__ int grow_expansion_zeroelim(double* e, int n, double 
 }
 
 // Exact sign of det[u, v, w] where u = b - a, v = c - a, w = d - a.
-__device__ __noinline__ int orient_exact(double ax, double ay, double az, double bx, double by,
-                                         double bz, double cx, double cy, double cz, double dx,
-                                         double dy, double dz) {
+__device__ __forceinline__ int orient_exact_inline(double ax, double ay, double az, double bx, double by,
+                                                   double bz, double cx, double cy, double cz, double dx,
+                                                   double dy, double dz) {
   double U[3][2], V[3][2], W[3][2];
   two_diff(bx, ax, U[0][0], U[0][1]);
   two_diff(by, ay, U[1][0], U[1][1]);
@@ -108,10 +108,17 @@ __device__ __noinline__ int orient_exact(double ax, double ay, double az, double
   return (top > 0.0) - (top < 0.0);
 }
 
-// Filtered exact orientation sign.
-__device__ __forceinline__ int orient_sign(double ax, double ay, double az, double bx, double by,
-                                           double bz, double cx, double cy, double cz, double dx,
-                                           double dy, double dz) {
+// The same behind a call.
+__device__ __noinline__ int orient_exact(double ax, double ay, double az, double bx, double by, double bz, double cx,
+                                         double cy, double cz, double dx, double dy, double dz) {
+  return orient_exact_inline(ax, ay, az, bx, by, bz, cx, cy, cz, dx, dy, dz);
+}
+
+// Filtered orientation sign: exact if not 0; 0 when the FP64 filter does not
+// certify one.
+__device__ __forceinline__ int orient_filter(double ax, double ay, double az, double bx, double by,
+                                             double bz, double cx, double cy, double cz, double dx,
+                                             double dy, double dz) {
   const double ux = __dsub_rn(bx, ax), uy = __dsub_rn(by, ay), uz = __dsub_rn(bz, az);
   const double vx = __dsub_rn(cx, ax), vy = __dsub_rn(cy, ay), vz = __dsub_rn(cz, az);
   const double wx = __dsub_rn(dx, ax), wy = __dsub_rn(dy, ay), wz = __dsub_rn(dz, az);
@@ -128,7 +135,15 @@ __device__ __forceinline__ int orient_sign(double ax, double ay, double az, doub
   const double bound = __dmul_rn((7.0 + 56.0 * eps) * eps, perm);
   if (det > bound) return 1;
   if (-det > bound) return -1;
-  return orient_exact(ax, ay, az, bx, by, bz, cx, cy, cz, dx, dy, dz);
+  return 0;
+}
+
+// Filtered exact orientation sign.
+__device__ __forceinline__ int orient_sign(double ax, double ay, double az, double bx, double by,
+                                           double bz, double cx, double cy, double cz, double dx,
+                                           double dy, double dz) {
+  const int s = orient_filter(ax, ay, az, bx, by, bz, cx, cy, cz, dx, dy, dz);
+  return s ? s : orient_exact(ax, ay, az, bx, by, bz, cx, cy, cz, dx, dy, dz);
 }
 
 // The FP32 stage alone: +1 or -1 when the FP32 filter certifies the sign, 0
