@@ -296,7 +296,6 @@ struct casim_sim {
   int2* cell_range = nullptr;
   int *pair_count = nullptr, *pair_tet = nullptr, *obs_sphere = nullptr, *int_of_user_d = nullptr;
   int* cast_list = nullptr;
-  double* cast_nrm = nullptr;
   double *knots_d = nullptr, *spheres_d = nullptr, *partials = nullptr, *e_partials = nullptr;
   float* spheres_fd = nullptr;
   SpringDev sp{};
@@ -520,7 +519,6 @@ Dev<T> make_dev(casim_sim* sim) {
   d.max_pairs = sim->params.max_pairs_per_vertex;
   d.sp = sim->sp;
   d.cast_list = sim->cast_list;
-  d.cast_nrm = sim->cast_nrm;
   d.spring_c = (R4<double>*)sim->spring_c;
   d.broad = sim->params.broad_phase;
   d.bt = sim->bt;
@@ -886,7 +884,6 @@ int upload_typed(casim_sim* sim, const std::vector<double>& rest_int, const std:
   sim->sp.target = sim->dalloc<double>(3 * (size_t)n_q);
   sim->sp.fallback = sim->dalloc<int>(n_q);
   sim->cast_list = sim->dalloc<int>(n_q);
-  sim->cast_nrm = sim->dalloc<double>(3 * (size_t)n_q);
   sim->int_of_user_d = sim->dalloc<int>(n_v);
   sim->robot_row = sim->dalloc<int>(sim->robot_row_h.size());
   sim->seg_d = sim->seg_blocks ? sim->dalloc<int>(sim->seg_h.size()) : nullptr;

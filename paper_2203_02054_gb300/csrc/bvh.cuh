@@ -135,96 +135,4 @@ __device__ __forceinline__ void bvh_point_query(const BvhDev& b, int tree, doubl
   }
 }
 
-// Nearest primitive: leaf(p) returns the primitive's squared distance (or a
-// negative value to skip it) and records it; bound() gives the best squared
-// distance so far.  A subtree is skipped only when its box is strictly
-// farther than the best, so equal distances still reach every candidate and
-// the caller's tie rule decides.
-template <typename Leaf, typename Bound>
-__device__ __forceinline__ void bvh_nearest(const BvhDev& b, int tree, double x, double y, double z, Leaf leaf,
-                                            Bound bound) {
-  if (b.n <= 0) return;
-  const int root = b.root ? b.root[tree] : 0;
-  if (root == BVH_EMPTY) return;
-  if (root < 0) {
-    leaf(~root);
-    return;
-  }
-  const PtF pf = pt_f(x, y, z);
-  int stack[BVH_STACK];
-  int sp = 0;
-  stack[sp++] = root;
-  while (sp > 0) {
-    const int node = stack[--sp];
-    if ((double)box_d2(b.lo[node], b.hi[node], pf) > bound()) continue;
-    const int2 c = b.child[node];
-    // visit the nearer child first (pushed last)
-    const int cs[2] = {c.x, c.y};
-    double dc[2];
-    for (int k = 0; k < 2; ++k) dc[k] = cs[k] < 0 ? 0.0 : (double)box_d2(b.lo[cs[k]], b.hi[cs[k]], pf);
-    const int first = dc[1] < dc[0] ? 1 : 0;
-    for (int j = 0; j < 2; ++j) {
-      const int k = j == 0 ? 1 - first : first;
-      const int ch = cs[k];
-      if (ch < 0) {
-        leaf(~ch);
-      } else if (dc[k] <= bound() && sp < BVH_STACK) {
-        stack[sp++] = ch;
-      }
-    }
-  }
-}
-
-// First hit along a ray: leaf(p) tests primitive p and records a hit; tbest()
-// gives the best ray parameter so far (+inf before any hit).  Boxes entered
-// beyond the best hit (with a relative margin) are skipped.
-template <typename Leaf, typename Best>
-__device__ __forceinline__ void bvh_ray(const BvhDev& b, int tree, const double (&o)[3], const double (&dir)[3],
-                                        Leaf leaf, Best tbest) {
-  if (b.n <= 0) return;
-  const int root = b.root ? b.root[tree] : 0;
-  if (root == BVH_EMPTY) return;
-  if (root < 0) {
-    leaf(~root);
-    return;
-  }
-  RayF r;
-  r.o = pt_f(o[0], o[1], o[2]);
-  for (int a = 0; a < 3; ++a) {
-    const float df = (float)dir[a];
-    r.inv[a] = df != 0.0f ? 1.0f / df : INFINITY;
-  }
-  int stack[BVH_STACK];
-  float node_t[BVH_STACK];  // entry parameter of each stacked node
-  int sp = 0;
-  const float t_root = ray_box_t(b.lo[root], b.hi[root], r);
-  if (t_root == INFINITY) return;
-  node_t[sp] = t_root;
-  stack[sp++] = root;
-  while (sp > 0) {
-    const int node = stack[--sp];
-    if ((double)node_t[sp] > tbest() * (1.0 + 1e-6) + 1e-9) continue;  // a nearer hit was found meanwhile
-    const int2 c = b.child[node];
-    const int cs[2] = {c.x, c.y};
-    float te[2];
-    for (int k = 0; k < 2; ++k) {
-      if (cs[k] < 0) {
-        leaf(~cs[k]);
-        te[k] = INFINITY;
-      } else {
-        te[k] = ray_box_t(b.lo[cs[k]], b.hi[cs[k]], r);
-      }
-    }
-    // push the farther child first, so the nearer one is visited next
-    const int nearer = te[1] < te[0] ? 1 : 0;
-    for (int j = 0; j < 2; ++j) {
-      const int k = j == 0 ? 1 - nearer : nearer;
-      if (cs[k] >= 0 && te[k] < INFINITY && (double)te[k] <= tbest() * (1.0 + 1e-6) + 1e-9 && sp < BVH_STACK) {
-        node_t[sp] = te[k];
-        stack[sp++] = cs[k];
-      }
-    }
-  }
-}
-
 }  // namespace casim

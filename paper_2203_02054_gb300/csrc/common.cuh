@@ -204,7 +204,6 @@ struct Dev {
   int max_pairs;
   SpringDev sp;
   int* cast_list;        // n_q: query indices whose spring needs a ray cast
-  double* cast_nrm;      // 3 n_q: unit vertex normal of each listed query vertex
   R4<double>* spring_c;  // n_free: (c, mask), FP64
   // AABB trees (broad phase 1) and the rigid tetrahedral obstacle
   int broad;             // 0 spatial hash, 1 AABB trees refitted every iteration
