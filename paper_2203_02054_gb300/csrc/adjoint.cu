@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(128) k_adj_local(Dev<T> d, AdjDev<T> a) {
       for (int j = 0; j < 3; ++j)
         D[i][j] = Xc[i][0] * Tm[j][0] + Xc[i][1] * Tm[j][1] + Xc[i][2] * Tm[j][2] + Xc[i][3] * Tm[j][3];
     T Rt[3][3], trt;
-    kabsch_rotation<T, SWEEPS>(D, Rt, trt);
+    rotation_fit<T, SWEEPS>(D, Rt, trt);
     // from here on FP64
     double R[3][3], X[3][4], Tc[3][4], RT[3][4];
     for (int i = 0; i < 3; ++i) {

@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(BS) k_local(Dev<T> d) {
       for (int j = 0; j < 3; ++j)
         D[i][j] = Xc[i][0] * Tm[j][0] + Xc[i][1] * Tm[j][1] + Xc[i][2] * Tm[j][2] + Xc[i][3] * Tm[j][3];
     T R[3][3], tr;
-    kabsch_rotation<T, SWEEPS>(D, R, tr);
+    rotation_fit<T, SWEEPS>(D, R, tr);
     T RT[3][4];
     for (int i = 0; i < 3; ++i)
       for (int k = 0; k < 4; ++k) RT[i][k] = R[i][0] * Tm[0][k] + R[i][1] * Tm[1][k] + R[i][2] * Tm[2][k];
