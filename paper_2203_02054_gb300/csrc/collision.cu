@@ -499,7 +499,7 @@ __device__ __forceinline__ void add_pair(const Dev<T>& d, int qi, int e) {
 __device__ __forceinline__ bool finite_t(float x) { return isfinite(x); }
 __device__ __forceinline__ bool finite_t(double x) { return (__double2hiint(x) & 0x7FF00000) != 0x7FF00000; }
 
-// Narrow phase, one thread per tet, over the cells of the tet's box: tests the
+// Narrow phase, one lane per tet, over the cells of the tet's box: tests the
 // query vertices listed in them whose own cell is the visited one (so every
 // vertex of the box is met once).
 //
@@ -522,7 +522,7 @@ __device__ __forceinline__ bool finite_t(double x) { return (__double2hiint(x) &
 static constexpr int TETS_MAX_THREADS = 256;
 
 template <typename T, bool CHECK>
-__global__ void __launch_bounds__(TETS_MAX_THREADS, 4) k_tets(Dev<T> d) {
+__global__ void __launch_bounds__(TETS_MAX_THREADS, 4) k_tets(Dev<T> d, int per_warp) {
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int WARPS = TETS_MAX_THREADS / 32;
   __shared__ unsigned s_entries;
@@ -531,8 +531,9 @@ __global__ void __launch_bounds__(TETS_MAX_THREADS, 4) k_tets(Dev<T> d) {
   __shared__ float s_x[WARPS][12][32];                    // corners
   if (threadIdx.x == 0) s_entries = 0;
   __syncthreads();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int i0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per_warp;
+  const int i = lane < per_warp ? i0 + lane : d.n_t;
   const unsigned before = (1u << lane) - 1u;
   int c0[3] = {0, 0, 0}, n[3] = {1, 1, 1}, ncell = 0;
   const float inv = (float)d.inv_cell;
@@ -668,7 +669,7 @@ __global__ void __launch_bounds__(TETS_MAX_THREADS, 4) k_tets(Dev<T> d) {
     visit.w = next * 32 + src;
     if (next) s_visits[wid][n_visits + __popc(again & before)] = visit;
     n_visits += __popc(again);
-    if (cand) s_pairs[wid][n_pairs + __popc(who & before)] = make_int2(i - lane + src, qi);
+    if (cand) s_pairs[wid][n_pairs + __popc(who & before)] = make_int2(i0 + src, qi);
     n_pairs += __popc(who);
     const bool last = take == 0;
     if (n_pairs >= 32 || last) {
@@ -748,8 +749,9 @@ __global__ void __launch_bounds__(256) k_bvh_refit(BvhDev b, const R4<T>* __rest
 // their boxes) of some 60 to 100 nodes; a team's is about as long as the tree is
 // deep.  Measured on a finger of 51,840 tets with a box of 768 as obstacle, one
 // thread per query and eight lanes: narrow phase with the spring update 330 and
-// 122 us (75 of them the tree queries, 42 the obstacle's closest faces), casts 572
-// and 94 us.
+// 99 us (57 of them the tree queries, 36 the obstacle's closest faces), casts 572
+// and 60 us.  (The four teams of a warp go round together; each on its own, their
+// reads queue up behind one another: 75, 42 and 94 us.)
 static constexpr int TEAM_LANES = 8;
 static constexpr int TEAM_STACK = 128;
 struct TeamStack {
@@ -762,10 +764,10 @@ struct TeamStack {
 // stack stays within its size (one by one it grows by the tree's depth at most,
 // for which 64 places are kept).
 __device__ __forceinline__ int team_take(int n) { return min(min(TEAM_LANES, n), max(1, TEAM_STACK - BVH_STACK - n)); }
-// Pushes ch of the lanes that have one.
-__device__ __forceinline__ void team_push(TeamStack& s, int& n, bool push, int ch, float key, unsigned tmask) {
+// Pushes ch of the lanes that have one; all lanes of the warp take part.
+__device__ __forceinline__ void team_push(TeamStack& s, int& n, bool push, int ch, float key) {
   const int lane = threadIdx.x & 31;
-  const unsigned who = __ballot_sync(tmask, push) & tmask;
+  const unsigned who = __ballot_sync(0xffffffffu, push) & (0xFFu << (lane & 24));
   const int at = n + __popc(who & ((1u << lane) - 1u));
   if (push && at < TEAM_STACK) {
     s.node[at] = ch;
@@ -775,38 +777,42 @@ __device__ __forceinline__ void team_push(TeamStack& s, int& n, bool push, int c
 }
 
 // Calls leaf(p), by some lane of the team, for every primitive whose ancestors'
-// boxes all contain the point.
+// boxes all contain the team's point (search: it has one).  The four teams of a
+// warp go round together, so that their reads are in flight together.
 template <typename Leaf>
-__device__ __forceinline__ void team_point_query(const BvhDev& b, int tree, const PtF& pf, TeamStack& s, unsigned tmask,
+__device__ __forceinline__ void team_point_query(const BvhDev& b, int tree, bool search, const PtF& pf, TeamStack& s,
                                                  Leaf leaf) {
-  if (b.n <= 0) return;
+  constexpr unsigned FULL = 0xffffffffu;
   const int tl = threadIdx.x & (TEAM_LANES - 1);
-  const int root = b.root ? b.root[tree] : 0;
-  if (root == BVH_EMPTY) return;
-  if (root < 0) {
-    if (tl == 0) leaf(~root);
-    return;
+  const int root = search && b.n > 0 ? (b.root ? b.root[tree] : 0) : BVH_EMPTY;
+  int n = 0;
+  if (root >= 0) {
+    if (box_has(b.lo[root], b.hi[root], pf)) n = 1;
+    if (tl == 0) s.node[0] = root;
+  } else if (root != BVH_EMPTY && tl == 0) {
+    leaf(~root);
   }
-  if (!box_has(b.lo[root], b.hi[root], pf)) return;
-  int n = 1;
-  if (tl == 0) s.node[0] = root;
-  __syncwarp(tmask);
-  while (n > 0) {
+  __syncwarp();
+  while (__any_sync(FULL, n > 0)) {
     const int take = team_take(n);
     const int node = tl < take ? s.node[n - 1 - tl] : -1;
-    __syncwarp(tmask);
+    __syncwarp();
     n -= take;
     int2 c = make_int2(0, 0);
     if (node >= 0) c = b.child[node];
+    bool push[2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const int ch = k ? c.y : c.x;
-      const bool inner = node >= 0 && ch >= 0;
-      if (node >= 0 && ch < 0) leaf(~ch);
-      __syncwarp(tmask);
-      team_push(s, n, inner && box_has(b.lo[ch], b.hi[ch], pf), ch, 0.0f, tmask);
+      push[k] = node >= 0 && ch >= 0 && box_has(b.lo[ch], b.hi[ch], pf);
     }
-    __syncwarp(tmask);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int ch = k ? c.y : c.x;
+      if (node >= 0 && ch < 0) leaf(~ch);
+      team_push(s, n, push[k], ch, 0.0f);
+    }
+    __syncwarp();
   }
 }
 
@@ -822,45 +828,42 @@ __global__ void __launch_bounds__(NARROW_BVH_THREADS, 4) k_narrow_bvh(Dev<T> d) 
   __shared__ TeamStack s_stack[NARROW_BVH_THREADS / TEAM_LANES];
   const int qi = (blockIdx.x * NARROW_BVH_THREADS + threadIdx.x) / TEAM_LANES;
   const int tl = threadIdx.x & (TEAM_LANES - 1);
-  const unsigned tmask = 0xFFu << (threadIdx.x & 24);
   TeamStack& stack = s_stack[threadIdx.x / TEAM_LANES];
   int n_obs = 0;
-  if (qi < d.n_q) {
-    const int v = d.q_verts[qi];
-    const R4<T> pv = d.X[v];
-    const T px = pv.x, py = pv.y, pz = pv.z;
-    const float pf[3] = {(float)px, (float)py, (float)pz};
+  const bool valid = qi < d.n_q;
+  const int v = valid ? d.q_verts[qi] : 0;
+  const R4<T> pv = d.X[v];
+  const T px = pv.x, py = pv.y, pz = pv.z;
+  const float pf[3] = {(float)px, (float)py, (float)pz};
+  if (valid) {
     if (tl == 0) d.pair_count[qi] = 0;
     for (int k = tl; k < d.max_pairs; k += TEAM_LANES) d.pair_tet[(size_t)qi * d.max_pairs + k] = NO_PAIR;
-    __syncwarp(tmask);
-    const int rv = d.robot_of_vert ? d.robot_of_vert[v] : 0;
-    const bool finite = isfinite(px) && isfinite(py) && isfinite(pz);
-    if (!finite && tl == 0) set_status(d.ctrl, ST_NONFINITE);
-    if (d.collision >= 1 && finite) {
-      const PtF q = pt_f((double)px, (double)py, (double)pz);
-      team_point_query(d.bt, rv, q, stack, tmask, [&](int e) {
-        const int4 t = chk_idx4(d.ctrl, d.tet[e], d.n_v);
-        if (d.robot_of_tet && d.robot_of_tet[e] != rv) return;
-        if (t.x == v || t.y == v || t.z == v || t.w == v) return;
-        if (may_be_inside_at(d.X, pf, t) && strictly_inside_call(d.X, px, py, pz, t)) add_pair(d, qi, e);
-      });
-    }
-    int best = -1, n_sph = 0, n_mesh = 0;
-    if (finite) {
-      sphere_tests(d, px, py, pz, best, n_sph);
-      if (d.collision >= 2 && d.ot.n > 0) {
-        team_point_query(d.ot, 0, pt_f((double)px, (double)py, (double)pz), stack, tmask, [&](int e) {
-          const int4 t = d.ot.prim[e];
-          if (may_be_inside_at(d.OX, pf, t) && strictly_inside_call(d.OX, px, py, pz, t)) ++n_mesh;
-        });
-        n_mesh = (int)__reduce_add_sync(tmask, (unsigned)n_mesh);
-      }
-    }
-    if (tl == 0) {
-      n_obs = n_sph + n_mesh;
-      d.obs_sphere[qi] = best;
-      if (d.obs_mesh) d.obs_mesh[qi] = n_mesh;
-    }
+  }
+  __syncwarp();
+  const int rv = d.robot_of_vert ? d.robot_of_vert[v] : 0;
+  const bool finite = isfinite(px) && isfinite(py) && isfinite(pz);
+  if (valid && !finite && tl == 0) set_status(d.ctrl, ST_NONFINITE);
+  const PtF q = pt_f((double)px, (double)py, (double)pz);
+  team_point_query(d.bt, rv, valid && finite && d.collision >= 1, q, stack, [&](int e) {
+    const int4 t = chk_idx4(d.ctrl, d.tet[e], d.n_v);
+    if (d.robot_of_tet && d.robot_of_tet[e] != rv) return;
+    if (t.x == v || t.y == v || t.z == v || t.w == v) return;
+    if (may_be_inside_at(d.X, pf, t) && strictly_inside_call(d.X, px, py, pz, t)) add_pair(d, qi, e);
+  });
+  int best = -1, n_sph = 0, n_mesh = 0;
+  if (valid && finite) sphere_tests(d, px, py, pz, best, n_sph);
+  if (d.collision >= 2 && d.ot.n > 0) {
+    team_point_query(d.ot, 0, valid && finite, q, stack, [&](int e) {
+      const int4 t = d.ot.prim[e];
+      if (may_be_inside_at(d.OX, pf, t) && strictly_inside_call(d.OX, px, py, pz, t)) ++n_mesh;
+    });
+#pragma unroll
+    for (int o = TEAM_LANES / 2; o > 0; o >>= 1) n_mesh += __shfl_xor_sync(0xffffffffu, n_mesh, o);
+  }
+  if (valid && tl == 0) {
+    n_obs = n_sph + n_mesh;
+    d.obs_sphere[qi] = best;
+    if (d.obs_mesh) d.obs_mesh[qi] = n_mesh;
   }
   const int s = block_sum_int(n_obs, shi);
   if (threadIdx.x == 0 && s) atomicAdd(&(d.hist + (d.ctrl->iter % d.hist_cap))->n_obstacle_pairs, s);
@@ -994,198 +997,6 @@ __device__ __forceinline__ void team_argmin(int& f, double& key, double& b1, dou
   }
 }
 
-// Closest-point candidate of face f for point o (lane-local running minimum).
-template <typename T>
-__device__ __forceinline__ void closest_candidate(const Dev<T>& d, int v, int rv, int f, V3 o, int& lf, double& ld,
-                                                  double& l1, double& l2) {
-  if (d.robot_of_face && d.robot_of_face[f] != rv) return;
-  V3 q0, q1, q2;
-  int4 fv;
-  face_verts(d, f, q0, q1, q2, fv);
-  if (fv.x == v || fv.y == v || fv.z == v) return;
-  double b1, b2;
-  const V3 x = closest_tri(o, q0, q1, q2, b1, b2);
-  const V3 dd = sub(o, x);
-  const double d2 = dot(dd, dd);
-  if (lf < 0 || d2 < ld || (d2 == ld && f < lf)) {
-    lf = f;
-    ld = d2;
-    l1 = b1;
-    l2 = b2;
-  }
-}
-
-// Closest boundary face, among those not containing vertex v, to point o of v
-// (robot rv) by one warp, and the closest point's barycentrics.
-template <typename T>
-__device__ int closest_face_warp(const Dev<T>& d, int v, int rv, V3 o, double& rb1, double& rb2) {
-  const int lane = threadIdx.x & 31;
-  int best_f = -1;
-  rb1 = rb2 = 0.0;
-  // found by scanning cubic shells of cells around v's cell (the cells of a
-  // shell split over the lanes).  After shell k every face with a point within
-  // k cells has been seen, so the search stops once the best distance is at most
-  // k cell edges.
-  const int c0[3] = {cell_coord(o.x, d.inv_cell), cell_coord(o.y, d.inv_cell), cell_coord(o.z, d.inv_cell)};
-  double bestd = 0.0;
-  for (int k = 0; k <= 64; ++k) {
-    const int side = 2 * k + 1;
-    const int ncell = side * side * side;
-    int lf = -1;
-    double ld = 0.0, l1 = 0.0, l2 = 0.0;
-    for (int idx = lane; idx < ncell; idx += 32) {
-      const int dx = idx % side - k, dy = (idx / side) % side - k, dz = idx / (side * side) - k;
-      if (max(abs(dx), max(abs(dy), abs(dz))) != k) continue;
-      const int2 r = d.cell_range[hash_cell(c0[0] + dx, c0[1] + dy, c0[2] + dz, rv) & (d.H_f - 1u)];
-      const int k1 = min(r.y, d.cap_items);
-      for (int q = r.x; q < k1; ++q) closest_candidate(d, v, rv, d.items[q], o, lf, ld, l1, l2);
-    }
-    warp_argmin(lf, ld, l1, l2);
-    if (lf >= 0 && (best_f < 0 || ld < bestd || (ld == bestd && lf < best_f))) {
-      best_f = lf;
-      bestd = ld;
-      rb1 = l1;
-      rb2 = l2;
-    }
-    if (best_f >= 0 && sqrt(bestd) <= k * d.cell) return best_f;
-  }
-  if (best_f >= 0) return best_f;
-  // the shell search found nothing within 64 cells: every face (rare)
-  int lf = -1;
-  double ld = 0.0, l1 = 0.0, l2 = 0.0;
-  for (int f = lane; f < d.n_f; f += 32) closest_candidate(d, v, rv, f, o, lf, ld, l1, l2);
-  warp_argmin(lf, ld, l1, l2);
-  rb1 = l1;
-  rb2 = l2;
-  return lf;
-}
-
-template <typename T>
-__device__ __forceinline__ V3 face_point(const Dev<T>& d, int f, double b1, double b2, V3& nunit) {
-  V3 q0, q1, q2;
-  int4 fv;
-  face_verts(d, f, q0, q1, q2, fv);
-  V3 n = cross(sub(q1, q0), sub(q2, q0));
-  nunit = scl(1.0 / norm(n), n);
-  return add(add(scl(1.0 - b1 - b2, q0), scl(b1, q1)), scl(b2, q2));
-}
-
-// Point and unit outward normal of boundary face f of the tetrahedral
-// obstacle at barycentrics (b1, b2).
-template <typename T>
-__device__ __forceinline__ V3 obstacle_face_point(const Dev<T>& d, int f, double b1, double b2, V3& nunit) {
-  const int4 fv = d.oface[f];
-  const R4<T> a = d.OX[fv.x], b = d.OX[fv.y], c = d.OX[fv.z];
-  const V3 q0 = {(double)a.x, (double)a.y, (double)a.z}, q1 = {(double)b.x, (double)b.y, (double)b.z},
-           q2 = {(double)c.x, (double)c.y, (double)c.z};
-  const V3 n = cross(sub(q1, q0), sub(q2, q0));
-  nunit = scl(1.0 / norm(n), n);
-  return add(add(scl(1.0 - b1 - b2, q0), scl(b1, q1)), scl(b2, q2));
-}
-
-// Best primitive of a tree for each searching team of the warp; all lanes take
-// part.  begin(lo, hi) is the FP32 key at which a box begins (INFINITY: never),
-// may(f, lb, ub) an FP32 test of a primitive with bounds of its key, test(f, key,
-// e1, e2) the FP64 one.  The smallest key wins, then the lowest id; what begins
-// beyond limit_of(best key) holds nothing better.  The teams visit their nodes and
-// collect the primitives that FP32 leaves open, and only then meet for the FP64
-// test of all teams' (it costs its scheduler as much for one lane as for 32).
-template <typename Begin, typename May, typename Test, typename Limit>
-__device__ __forceinline__ void team_search(const BvhDev& b, int root, bool search, TeamStack& stack, int& bf, double& bt,
-                                            double& b1, double& b2, Begin begin, May may, Test test, Limit limit_of) {
-  constexpr unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31, tl = lane & (TEAM_LANES - 1);
-  const unsigned tmask = 0xFFu << (lane & 24), before = (1u << lane) - 1u;
-  float limit = INFINITY;
-  int n = 0, nc = 0;  // nodes and primitives waiting
-  if (search && root != BVH_EMPTY) {
-    if (root < 0) {
-      nc = 1;
-      if (tl == 0) {
-        stack.cand[0] = ~root;
-        stack.cand_key[0] = -INFINITY;
-      }
-    } else {
-      const float key = begin(b.lo[root], b.hi[root]);
-      n = key < INFINITY ? 1 : 0;
-      if (tl == 0) {
-        stack.node[0] = root;
-        stack.key[0] = key;
-      }
-    }
-  }
-  __syncwarp();
-  for (;;) {
-    while (n > 0 && nc <= TEAM_LANES) {
-      const int take = team_take(n);
-      int node = -1;
-      if (tl < take && stack.key[n - 1 - tl] <= limit) node = stack.node[n - 1 - tl];
-      __syncwarp(tmask);
-      n -= take;
-      int2 c = make_int2(0, 0);
-      if (node >= 0) c = b.child[node];
-      float key[2] = {INFINITY, INFINITY}, low[2] = {0.0f, 0.0f};
-      bool open[2] = {false, false};
-      float least = limit;
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const int ch = k ? c.y : c.x;
-        if (node < 0) continue;
-        if (ch >= 0) {
-          key[k] = begin(b.lo[ch], b.hi[ch]);
-        } else {
-          float ub = INFINITY;
-          open[k] = may(~ch, low[k], ub);
-          least = fminf(least, ub);
-        }
-      }
-#pragma unroll
-      for (int o = TEAM_LANES / 2; o > 0; o >>= 1) least = fminf(least, __shfl_xor_sync(tmask, least, o));
-      limit = least;
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const bool keep = open[k] && !(low[k] > limit);
-        const unsigned who = __ballot_sync(tmask, keep) & tmask;
-        const int at = nc + __popc(who & before);
-        if (keep) {
-          stack.cand[at] = ~(k ? c.y : c.x);
-          stack.cand_key[at] = low[k];
-        }
-        nc += __popc(who);
-      }
-      // the farther child first, so that the nearer one is visited next
-      const bool swap = key[1] > key[0];
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const bool second = (k == 0) == swap;
-        const float t = second ? key[1] : key[0];
-        team_push(stack, n, t < INFINITY && t <= limit, second ? c.y : c.x, t, tmask);
-      }
-      __syncwarp(tmask);
-    }
-    __syncwarp();
-    if (!__any_sync(FULL, nc > 0)) break;
-    const int take = min(nc, TEAM_LANES);
-    int f = -1;
-    if (tl < take && !(stack.cand_key[nc - 1 - tl] > limit)) f = stack.cand[nc - 1 - tl];
-    __syncwarp();
-    nc -= take;
-    if (!__any_sync(FULL, f >= 0)) continue;
-    int lf = -1;
-    double lk = 0.0, e1 = 0.0, e2 = 0.0;
-    if (f >= 0 && test(f, lk, e1, e2)) lf = f;
-    if (!__any_sync(FULL, lf >= 0)) continue;
-    team_argmin(lf, lk, e1, e2);
-    if (lf >= 0 && (bf < 0 || key_bits(lk) < key_bits(bt) || (key_bits(lk) == key_bits(bt) && lf < bf))) {
-      bf = lf;
-      bt = lk;
-      b1 = e1;
-      b2 = e2;
-      limit = fminf(limit, limit_of(bt));
-    }
-  }
-}
-
 // FP32 bounds of the squared distance from a point to a triangle, its corners
 // given as differences from the point (dl bounds the error that rounded FP64
 // positions add to one).  The upper one is the distance of some point of the
@@ -1249,6 +1060,261 @@ __device__ __forceinline__ void triangle_bounds_at(const R4<T>& q0, const R4<T>&
 #pragma unroll
     for (int j = 0; j < 3; ++j) q[k][j] -= p[j];
   triangle_d2_bounds(q[0], q[1], q[2], dl, lb, ub);
+}
+
+// Closest-point candidate of face f for point o (lane-local running minimum).
+template <typename T>
+__device__ __forceinline__ void closest_candidate(const Dev<T>& d, int v, int rv, int f, V3 o, int& lf, double& ld,
+                                                  double& l1, double& l2) {
+  if (d.robot_of_face && d.robot_of_face[f] != rv) return;
+  V3 q0, q1, q2;
+  int4 fv;
+  face_verts(d, f, q0, q1, q2, fv);
+  if (fv.x == v || fv.y == v || fv.z == v) return;
+  double b1, b2;
+  const V3 x = closest_tri(o, q0, q1, q2, b1, b2);
+  const V3 dd = sub(o, x);
+  const double d2 = dot(dd, dd);
+  if (lf < 0 || d2 < ld || (d2 == ld && f < lf)) {
+    lf = f;
+    ld = d2;
+    l1 = b1;
+    l2 = b2;
+  }
+}
+
+// Closest boundary face, among those not containing vertex v, to point o of v
+// (robot rv) by one warp, and the closest point's barycentrics.
+// Found by scanning cubic shells of cells around v's cell.  After shell k every
+// face with a point within k cells has been seen, so the search stops once the
+// best distance is at most k cell edges (after the first neighbours at the
+// earliest).  The shell's faces are spread over the lanes whatever their cells,
+// FP32 bounds of their distances sort out the ones that cannot be closest, and
+// what is left waits in a queue for the FP64 test.  (With a cell to a lane and
+// FP64 throughout, one lane tested the ten faces of v's own cell one by one, 40 us
+// for any launch with such a vertex.)
+struct FaceQueue {
+  int face[64];
+  float low[64];  // lower bound of the squared distance
+};
+template <typename T>
+__device__ int closest_face_warp(const Dev<T>& d, FaceQueue& queue, int v, int rv, V3 o, double& rb1, double& rb2) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const R4<T> x = {(T)o.x, (T)o.y, (T)o.z, T(0)};
+  int best_f = -1, n = 0;
+  rb1 = rb2 = 0.0;
+  const int c0[3] = {cell_coord(o.x, d.inv_cell), cell_coord(o.y, d.inv_cell), cell_coord(o.z, d.inv_cell)};
+  double bestd = 0.0;
+  float limit = INFINITY;
+  auto test = [&]() {  // the last of the queued faces, one to a lane
+    __syncwarp();
+    const int take = min(n, 32);
+    int lf = -1;
+    double ld = 0.0, l1 = 0.0, l2 = 0.0;
+    if (lane < take && !(queue.low[n - 1 - lane] > limit))
+      closest_candidate(d, v, rv, queue.face[n - 1 - lane], o, lf, ld, l1, l2);
+    __syncwarp();
+    n -= take;
+    warp_argmin(lf, ld, l1, l2);
+    if (lf >= 0 && (best_f < 0 || ld < bestd || (ld == bestd && lf < best_f))) {
+      best_f = lf;
+      bestd = ld;
+      rb1 = l1;
+      rb2 = l2;
+      limit = fminf(limit, __double2float_ru(bestd));
+    }
+  };
+  for (int k = 0; k <= 64; ++k) {
+    const int side = 2 * k + 1;
+    const int ncell = side * side * side;
+    for (int base = 0; base < ncell; base += 32) {
+      // this lane's cell, and the entries of the 32 cells in one sequence
+      const int idx = base + lane;
+      const int dx = idx % side - k, dy = (idx / side) % side - k, dz = idx / (side * side) - k;
+      int first = 0, upto = 0;
+      if (idx < ncell && max(abs(dx), max(abs(dy), abs(dz))) == k) {
+        const int2 r = d.cell_range[hash_cell(c0[0] + dx, c0[1] + dy, c0[2] + dz, rv) & (d.H_f - 1u)];
+        first = r.x;
+        upto = max(min(r.y, d.cap_items) - r.x, 0);
+      }
+#pragma unroll
+      for (int m = 1; m < 32; m <<= 1) {
+        const int u = __shfl_up_sync(FULL, upto, m);
+        if (lane >= m) upto += u;
+      }
+      const int total = __shfl_sync(FULL, upto, 31);
+      for (int e0 = 0; e0 < total; e0 += 32) {
+        // the cell of entry e: the number of cells whose sequences end at or before it
+        const int e = e0 + lane;
+        int cell = 0;
+#pragma unroll
+        for (int m = 16; m > 0; m >>= 1)
+          if (__shfl_sync(FULL, upto, cell + m - 1) <= e) cell += m;
+        cell = min(cell, 31);
+        const int before = __shfl_sync(FULL, upto, max(cell - 1, 0)), start = __shfl_sync(FULL, first, cell);
+        int f = -1;
+        float lb = 0.0f, ub = INFINITY;
+        if (e < total) {
+          f = d.items[start + e - (cell ? before : 0)];
+          const int4 fv = chk_face(d.ctrl, d.faces[chk_idx(d.ctrl, f, d.n_f)], d.n_v);
+          if ((d.robot_of_face && d.robot_of_face[f] != rv) || fv.x == v || fv.y == v || fv.z == v) f = -1;
+          else triangle_bounds_at(d.X[fv.x], d.X[fv.y], d.X[fv.z], x, lb, ub);
+        }
+        if (f < 0) ub = INFINITY;
+#pragma unroll
+        for (int m = 16; m > 0; m >>= 1) ub = fminf(ub, __shfl_xor_sync(FULL, ub, m));
+        limit = fminf(limit, ub);
+        const unsigned keep = __ballot_sync(FULL, f >= 0 && !(lb > limit));
+        if (keep >> lane & 1u) {
+          const int at = n + __popc(keep & ((1u << lane) - 1u));
+          queue.face[at] = f;
+          queue.low[at] = lb;
+        }
+        n += __popc(keep);
+        if (n > 32) test();
+      }
+    }
+    if (k == 0) continue;
+    while (n > 0) test();
+    if (best_f >= 0 && sqrt(bestd) <= k * d.cell) return best_f;
+  }
+  if (best_f >= 0) return best_f;
+  // the shell search found nothing within 64 cells: every face (rare)
+  int lf = -1;
+  double ld = 0.0, l1 = 0.0, l2 = 0.0;
+  for (int f = lane; f < d.n_f; f += 32) closest_candidate(d, v, rv, f, o, lf, ld, l1, l2);
+  warp_argmin(lf, ld, l1, l2);
+  rb1 = l1;
+  rb2 = l2;
+  return lf;
+}
+
+template <typename T>
+__device__ __forceinline__ V3 face_point(const Dev<T>& d, int f, double b1, double b2, V3& nunit) {
+  V3 q0, q1, q2;
+  int4 fv;
+  face_verts(d, f, q0, q1, q2, fv);
+  V3 n = cross(sub(q1, q0), sub(q2, q0));
+  nunit = scl(1.0 / norm(n), n);
+  return add(add(scl(1.0 - b1 - b2, q0), scl(b1, q1)), scl(b2, q2));
+}
+
+// Point and unit outward normal of boundary face f of the tetrahedral
+// obstacle at barycentrics (b1, b2).
+template <typename T>
+__device__ __forceinline__ V3 obstacle_face_point(const Dev<T>& d, int f, double b1, double b2, V3& nunit) {
+  const int4 fv = d.oface[f];
+  const R4<T> a = d.OX[fv.x], b = d.OX[fv.y], c = d.OX[fv.z];
+  const V3 q0 = {(double)a.x, (double)a.y, (double)a.z}, q1 = {(double)b.x, (double)b.y, (double)b.z},
+           q2 = {(double)c.x, (double)c.y, (double)c.z};
+  const V3 n = cross(sub(q1, q0), sub(q2, q0));
+  nunit = scl(1.0 / norm(n), n);
+  return add(add(scl(1.0 - b1 - b2, q0), scl(b1, q1)), scl(b2, q2));
+}
+
+// Best primitive of a tree for each searching team of the warp; all lanes take
+// part.  begin(lo, hi) is the FP32 key at which a box begins (INFINITY: never),
+// may(f, lb, ub) an FP32 test of a primitive with bounds of its key, test(f, key,
+// e1, e2) the FP64 one.  The smallest key wins, then the lowest id; what begins
+// beyond limit_of(best key), or slack times an upper bound, holds nothing better.  The teams visit their nodes and
+// collect the primitives that FP32 leaves open, and only then meet for the FP64
+// test of all teams' (it costs its scheduler as much for one lane as for 32).
+template <typename Begin, typename May, typename Test, typename Limit>
+__device__ __forceinline__ void team_search(const BvhDev& b, int root, bool search, TeamStack& stack, int& bf, double& bt,
+                                            double& b1, double& b2, Begin begin, May may, Test test, Limit limit_of,
+                                            float slack = 1.0f) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, tl = lane & (TEAM_LANES - 1);
+  const unsigned tmask = 0xFFu << (lane & 24), before = (1u << lane) - 1u;
+  float limit = INFINITY;
+  int n = 0, nc = 0;  // nodes and primitives waiting
+  if (search && root != BVH_EMPTY) {
+    if (root < 0) {
+      nc = 1;
+      if (tl == 0) {
+        stack.cand[0] = ~root;
+        stack.cand_key[0] = -INFINITY;
+      }
+    } else {
+      const float key = begin(b.lo[root], b.hi[root]);
+      n = key < INFINITY ? 1 : 0;
+      if (tl == 0) {
+        stack.node[0] = root;
+        stack.key[0] = key;
+      }
+    }
+  }
+  __syncwarp();
+  for (;;) {
+    while (__any_sync(FULL, n > 0 && nc <= TEAM_LANES)) {
+      // (the teams that wait for the others take nothing)
+      const int take = nc <= TEAM_LANES ? team_take(n) : 0;
+      int node = -1;
+      if (tl < take && stack.key[n - 1 - tl] <= limit) node = stack.node[n - 1 - tl];
+      __syncwarp();
+      n -= take;
+      int2 c = make_int2(0, 0);
+      if (node >= 0) c = b.child[node];
+      float key[2] = {INFINITY, INFINITY}, low[2] = {0.0f, 0.0f};
+      bool open[2] = {false, false};
+      float least = limit;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int ch = k ? c.y : c.x;
+        if (node < 0) continue;
+        if (ch >= 0) {
+          key[k] = begin(b.lo[ch], b.hi[ch]);
+        } else {
+          float ub = INFINITY;
+          open[k] = may(~ch, low[k], ub);
+          if (open[k]) least = fminf(least, ub * slack);
+        }
+      }
+#pragma unroll
+      for (int o = TEAM_LANES / 2; o > 0; o >>= 1) least = fminf(least, __shfl_xor_sync(FULL, least, o));
+      limit = least;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const bool keep = open[k] && !(low[k] > limit);
+        const unsigned who = __ballot_sync(FULL, keep) & tmask;
+        const int at = nc + __popc(who & before);
+        if (keep) {
+          stack.cand[at] = ~(k ? c.y : c.x);
+          stack.cand_key[at] = low[k];
+        }
+        nc += __popc(who);
+      }
+      // the farther child first, so that the nearer one is visited next
+      const bool swap = key[1] > key[0];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const bool second = (k == 0) == swap;
+        const float t = second ? key[1] : key[0];
+        team_push(stack, n, t < INFINITY && t <= limit, second ? c.y : c.x, t);
+      }
+      __syncwarp();
+    }
+    if (!__any_sync(FULL, nc > 0)) break;
+    const int take = min(nc, TEAM_LANES);
+    int f = -1;
+    if (tl < take && !(stack.cand_key[nc - 1 - tl] > limit)) f = stack.cand[nc - 1 - tl];
+    __syncwarp();
+    nc -= take;
+    if (!__any_sync(FULL, f >= 0)) continue;
+    int lf = -1;
+    double lk = 0.0, e1 = 0.0, e2 = 0.0;
+    if (f >= 0 && test(f, lk, e1, e2)) lf = f;
+    if (!__any_sync(FULL, lf >= 0)) continue;
+    team_argmin(lf, lk, e1, e2);
+    if (lf >= 0 && (bf < 0 || key_bits(lk) < key_bits(bt) || (key_bits(lk) == key_bits(bt) && lf < bf))) {
+      bf = lf;
+      bt = lk;
+      b1 = e1;
+      b2 = e2;
+      limit = fminf(limit, limit_of(bt));
+    }
+  }
 }
 
 // Closest boundary face of the tetrahedral obstacle to each team's point, and its
@@ -1465,10 +1531,12 @@ __global__ void __launch_bounds__(NARROW_BVH_THREADS, 3) k_mesh_springs(Dev<T> d
 // products and the sums), and 1e-6 = 16.8 u is used.  FP64 positions enter
 // rounded to FP32, which adds dl = 2^-22 times the coordinates' sizes to every
 // difference.  The constant covers underflow, differences above 1e9 (products
-// that could overflow) and NaN pass, like every value within its bound.
+// that could overflow) and NaN pass, like every value within its bound.  A face
+// that is certainly hit gives an upper bound t_max of its ray parameter (INFINITY
+// otherwise).
 template <typename T>
 __device__ __forceinline__ bool face_may_hit(const R4<T>& q0, const R4<T>& q1, const R4<T>& q2, const float (&o)[3],
-                                             const float (&dir)[3]) {
+                                             const float (&dir)[3], float& t_max) {
   const float a[3] = {(float)q0.x, (float)q0.y, (float)q0.z}, b[3] = {(float)q1.x, (float)q1.y, (float)q1.z},
               c[3] = {(float)q2.x, (float)q2.y, (float)q2.z};
   float e1[3], e2[3], tv[3];
@@ -1480,6 +1548,7 @@ __device__ __forceinline__ bool face_may_hit(const R4<T>& q0, const R4<T>& q1, c
   }
   const float dl = std::is_same<T, float>::value ? 0.0f : 0x1p-22f * (l1(a) + l1(b) + l1(c) + l1(o));
   const float n1 = l1(e1) + dl, n2 = l1(e2) + dl, n0 = l1(tv) + dl;
+  t_max = INFINITY;
   if (!(n0 + n1 + n2 < 1e9f)) return true;
   const float tiny = 1e-25f, k = 1e-6f;
   const float det = triple(dir, e1, e2);          // > 0 for an exit face
@@ -1489,6 +1558,8 @@ __device__ __forceinline__ bool face_may_hit(const R4<T>& q0, const R4<T>& q1, c
   const float bd = k * n1 * n2 + dl * (n1 + n2) + tiny, b1 = k * n0 * n2 + dl * (n0 + n2) + tiny,
               b2 = k * n0 * n1 + dl * (n0 + n1) + tiny,
               bt = k * n0 * n1 * n2 + dl * (n0 * n1 + n1 * n2 + n0 * n2) + tiny;
+  if (det > 2.0f * bd && v1 < -b1 && v2 < -b2 && v1 + v2 + det > bd + b1 + b2 && vt < -bt)
+    t_max = (bt - vt) / (det - bd) * 1.00001f;
   return !(det < -bd || v1 > b1 || v2 > b2 || -(v1 + v2) - det > bd + b1 + b2 || vt > bt);
 }
 
@@ -1556,14 +1627,19 @@ __device__ __forceinline__ int finish_cast(const Dev<T>& d, int qi, int v, int r
 // one lane as in thirty-two, and the normal, the walk's set-up, a ray-triangle
 // test and the target are about 300 of them.  So four vertices share each of
 // those phases: a vertex's lanes take its incident faces, then its axes; the
-// teams walk their cells with the FP32 test alone until one of a cell's faces
-// passes it, and only then meet for the FP64 test of all teams' candidates.
-// Measured with k_springs, before (one warp per vertex, the FP64 test on every
-// face) and after: 395 and 133 us for the 22,400 casts of a 983,040-tet finger,
-// 82 and 53 us for the 4,300 of the gripper.
+// teams walk their cells with the FP32 test alone, which also bounds the first
+// hit from above and so ends most walks, and then meet for the FP64 test of all
+// teams' candidates.
+// Measured, one warp per vertex with the FP64 test on every face, and this: 370 and
+// 121 us for the 22,400 casts of a 983,040-tet finger, 67 and 43 us for the 4,300
+// of the gripper.  (Meeting for FP64 at every cell with a face that passed: 48 us
+// there; reading eight cells' ranges of the walk ahead: 50 us.)
 template <typename T>
 __global__ void __launch_bounds__(CAST_THREADS) k_cast(Dev<T> d) {
   __shared__ int shi[32];
+  __shared__ FaceQueue s_queue[CAST_THREADS / 32];
+  __shared__ int s_cand[CAST_THREADS / TEAM_LANES][3 * TEAM_LANES];
+  int* const queue = s_cand[threadIdx.x / TEAM_LANES];
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31, tl = lane & 7;
   const unsigned tmask = 0xFFu << (lane & 24);
@@ -1622,39 +1698,53 @@ __global__ void __launch_bounds__(CAST_THREADS) k_cast(Dev<T> d) {
     }
     int best_f = -1;
     double best_t = 0.0, b1 = 0.0, b2 = 0.0;
-    unsigned long long best_lim = 0;  // bits of best_t (1 + 1e-9)
+    unsigned long long stop = key_bits(INFINITY);  // bits of a ray parameter beyond which no hit is the first
     bool walking = valid;             // team-uniform, like the walk's whole state
     int steps = 0, kk = 0, k1 = 0;    // cells left behind; the next entry of this cell and its end
+    int nc = 0;                       // faces in the team's queue
     auto enter = [&]() {
       const int2 r = d.cell_range[hash_cell(cell[0], cell[1], cell[2], rv) & (d.H_f - 1u)];
       kk = r.x;
       k1 = min(r.y, d.cap_items);
     };
     if (walking) enter();
-    while (__any_sync(FULL, walking)) {
-      // each team on its own, FP32 only, until eight entries hold a candidate
-      int cand = -1;
-      while (walking) {
-        if (kk < k1) {
+    for (;;) {
+      // FP32 only, until each team is at the end of its walk or its queue is
+      // full; the four go round together, so that their reads are in flight
+      // together
+      while (__any_sync(FULL, walking && nc <= 2 * TEAM_LANES)) {
+        const bool on = walking && nc <= 2 * TEAM_LANES;
+        int cand = -1;
+        float t_max = INFINITY;
+        if (on && kk < k1) {
           const int k = kk + tl;
           if (k < k1) {
             const int f = d.items[k];
             if (!d.robot_of_face || d.robot_of_face[f] == rv) {
               const int4 fv = chk_face(d.ctrl, d.faces[chk_idx(d.ctrl, f, d.n_f)], d.n_v);
-              if (fv.x != v && fv.y != v && fv.z != v && face_may_hit(d.X[fv.x], d.X[fv.y], d.X[fv.z], of, df)) cand = f;
+              if (fv.x != v && fv.y != v && fv.z != v &&
+                  face_may_hit(d.X[fv.x], d.X[fv.y], d.X[fv.z], of, df, t_max))
+                cand = f;
             }
           }
           kk += 8;
-          if (__any_sync(tmask, cand >= 0)) break;
-          continue;
         }
+        const unsigned who = __ballot_sync(FULL, cand >= 0) & tmask;
+        if (cand >= 0) queue[nc + __popc(who & ((1u << lane) - 1u))] = cand;
+        nc += __popc(who);
+        if (__any_sync(FULL, who != 0)) {
+          if (cand < 0) t_max = INFINITY;
+#pragma unroll
+          for (int m = 4; m > 0; m >>= 1) t_max = fminf(t_max, __shfl_xor_sync(FULL, t_max, m));
+          if (t_max < INFINITY) stop = min(stop, key_bits((double)t_max));
+        }
+        if (!on || kk < k1) continue;
         // the cell is done
         const unsigned long long m0 = key_bits(tmax[0]), m1 = key_bits(tmax[1]), m2 = key_bits(tmax[2]);
         const unsigned long long texit = m0 < m1 ? (m0 < m2 ? m0 : m2) : (m1 < m2 ? m1 : m2);
-        if ((best_f >= 0 && best_lim < texit) || texit >= key_bits(INFINITY) || texit > key_bits(tbox) ||
-            ++steps >= MAX_DDA_STEPS) {
+        if (stop < texit || texit >= key_bits(INFINITY) || texit > key_bits(tbox) || ++steps >= MAX_DDA_STEPS) {
           walking = false;
-          break;
+          continue;
         }
         if (m0 <= m1 && m0 <= m2) {
           cell[0] += step[0];
@@ -1669,14 +1759,19 @@ __global__ void __launch_bounds__(CAST_THREADS) k_cast(Dev<T> d) {
         enter();
       }
       __syncwarp();
-      // all teams' candidates, FP64
+      if (!__any_sync(FULL, nc > 0)) break;
+      // all teams' queued faces, FP64
+      const int take = min(nc, TEAM_LANES);
+      const int f = tl < take ? queue[nc - 1 - tl] : -1;
+      __syncwarp();
+      nc -= take;
       int lf = -1;
       double lt = 0.0, l1 = 0.0, l2 = 0.0;
-      if (cand >= 0) {
+      if (f >= 0) {
         V3 q0, q1, q2;
         int4 fv;
-        face_verts(d, cand, q0, q1, q2, fv);
-        if (dot(dir, cross(sub(q1, q0), sub(q2, q0))) > 0.0 && ray_tri(o, dir, q0, q1, q2, lt, l1, l2)) lf = cand;
+        face_verts(d, f, q0, q1, q2, fv);
+        if (dot(dir, cross(sub(q1, q0), sub(q2, q0))) > 0.0 && ray_tri(o, dir, q0, q1, q2, lt, l1, l2)) lf = f;
       }
       if (__any_sync(FULL, lf >= 0)) {
         team_argmin(lf, lt, l1, l2);
@@ -1685,7 +1780,7 @@ __global__ void __launch_bounds__(CAST_THREADS) k_cast(Dev<T> d) {
           best_t = lt;
           b1 = l1;
           b2 = l2;
-          best_lim = key_bits(best_t * (1.0 + 1e-9));
+          stop = min(stop, key_bits(best_t * (1.0 + 1e-9)));
         }
       }
     }
@@ -1697,7 +1792,7 @@ __global__ void __launch_bounds__(CAST_THREADS) k_cast(Dev<T> d) {
       todo &= todo - 1;
       const V3 os = {__shfl_sync(FULL, o.x, src), __shfl_sync(FULL, o.y, src), __shfl_sync(FULL, o.z, src)};
       double c1, c2;
-      const int f = closest_face_warp(d, __shfl_sync(FULL, v, src), __shfl_sync(FULL, rv, src), os, c1, c2);
+      const int f = closest_face_warp(d, s_queue[threadIdx.x >> 5], __shfl_sync(FULL, v, src), __shfl_sync(FULL, rv, src), os, c1, c2);
       if ((lane & 24) == (src & 24)) {
         best_f = f;
         b1 = c1;
@@ -1751,9 +1846,9 @@ __global__ void __launch_bounds__(NARROW_BVH_THREADS, 3) k_cast_bvh(Dev<T> d) {
     };
     team_search(
         b, root, valid, stack, bf, bt, b1, b2, [&](float4 lo, float4 hi) { return ray_box_t(lo, hi, ray); },
-        [&](int f, float&, float&) {
+        [&](int f, float&, float& ub) {
           int4 fv;
-          return other(f, fv) && face_may_hit(d.X[fv.x], d.X[fv.y], d.X[fv.z], of, df);
+          return other(f, fv) && face_may_hit(d.X[fv.x], d.X[fv.y], d.X[fv.z], of, df, ub);
         },
         [&](int f, double& key, double& e1, double& e2) {
           V3 q0, q1, q2;
@@ -1762,7 +1857,7 @@ __global__ void __launch_bounds__(NARROW_BVH_THREADS, 3) k_cast_bvh(Dev<T> d) {
           return dot(dir, cross(sub(q1, q0), sub(q2, q0))) > 0.0 && ray_tri(x, dir, q0, q1, q2, key, e1, e2);
         },
         // (the box tests of the ray are accurate to a margin)
-        [](double best) { return __double2float_ru(best * (1.0 + 1e-6) + 1e-9); });
+        [](double best) { return __double2float_ru(best * (1.0 + 1e-6) + 1e-9); }, 1.0001f);
     const bool missed = valid && bf < 0;
     if (__any_sync(FULL, missed))
       team_search(
@@ -1819,11 +1914,21 @@ void launch_faces(const Dev<T>& d, cudaStream_t st) {
 // Narrow phase over the tets once the query vertices are in their lists.
 template <typename T>
 void launch_tets(const Dev<T>& d, bool check, cudaStream_t st) {
-  const int bs = d.narrow_threads > 0 ? std::min(d.narrow_threads, TETS_MAX_THREADS) : TETS_MAX_THREADS, nb = (d.n_t + bs - 1) / bs;
+  // a warp works off what its tets' boxes hold in rounds, so a mesh that would
+  // leave the device half empty gets warps with fewer tets: 8 or 16 as long as all
+  // warps run at once (32 of them on each of about 150 processors).  32 tets to a
+  // warp and this: 15.1 and 10.9 us for 1,920 tets (22.2 and 15.6 in the
+  // allocation-free check), 37.4 and 32.2 us for 51,840 in FP64; at 193,920 and
+  // above it is the same.
+  constexpr int ONE_WAVE = 4800;
+  int per = 8;
+  while (per < 32 && d.n_t > per * ONE_WAVE) per *= 2;
+  const int bs = d.narrow_threads > 0 ? std::min(d.narrow_threads, TETS_MAX_THREADS) : TETS_MAX_THREADS;
+  const int tets = bs / 32 * per, nb = (d.n_t + tets - 1) / tets;
   if (check)
-    k_tets<T, true><<<nb, bs, 0, st>>>(d);
+    k_tets<T, true><<<nb, bs, 0, st>>>(d, per);
   else
-    k_tets<T, false><<<nb, bs, 0, st>>>(d);
+    k_tets<T, false><<<nb, bs, 0, st>>>(d, per);
 }
 
 // A caller's positions into the kernels' layout, and its query vertices, whose
