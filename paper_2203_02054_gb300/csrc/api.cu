@@ -1392,6 +1392,15 @@ int forward_ckpt_typed(casim_sim* sim, int n_iters, int every) {
 
 template <typename T>
 int backward_typed(casim_sim* sim, const double* dL_dX, double* dL_dalpha) {
+  // The pass is linear in dL_dX, and a MIXED one solves in FP32 with squared
+  // residuals: bring the largest entry to [1, 2) by a power of two (exact), so
+  // that a loss in any units meets the same range.
+  double unit = 1.0;
+  if (std::is_same<T, float>::value) {
+    double m = 0.0;
+    for (size_t k = 0; k < 3 * (size_t)sim->n_v; ++k) m = std::max(m, std::fabs(dL_dX[k]));
+    if (m > 1e-250 && m < 1e250) unit = std::ldexp(1.0, -std::ilogb(m));
+  }
   auto& A = sim->adj;
   cudaStream_t st = sim->stream;
   const size_t nv = sim->n_v, nq = std::max(sim->n_q, 1);
@@ -1400,7 +1409,8 @@ int backward_typed(casim_sim* sim, const double* dL_dX, double* dL_dalpha) {
   std::vector<R4<double>> gh(std::max(nf, 1));
   for (int uv = 0; uv < sim->n_v; ++uv) {
     const int i = sim->int_of_user[uv];
-    if (i < nf) gh[i] = R4<double>{dL_dX[3 * (size_t)uv], dL_dX[3 * (size_t)uv + 1], dL_dX[3 * (size_t)uv + 2], 0.0};
+    if (i < nf)
+      gh[i] = R4<double>{unit * dL_dX[3 * (size_t)uv], unit * dL_dX[3 * (size_t)uv + 1], unit * dL_dX[3 * (size_t)uv + 2], 0.0};
   }
   CK(cudaMemcpyAsync(A.g, gh.data(), sizeof(R4<double>) * std::max(nf, 1), cudaMemcpyHostToDevice, st));
   CK(cudaMemsetAsync(A.abar, 0, sizeof(double) * std::max(ng, 1), st));
@@ -1494,7 +1504,7 @@ int backward_typed(casim_sim* sim, const double* dL_dX, double* dL_dalpha) {
   CK(cudaMemcpy(sim->ctrl, &saved, sizeof(Ctrl), cudaMemcpyHostToDevice));
   // the recomputation used the history slots from here on: clear the next one
   CK(cudaMemset(sim->hist + (saved.iter % sim->hist_cap), 0, sizeof(IterRec)));
-  for (int gi = 0; gi < ng; ++gi) dL_dalpha[gi] = ab[gi];
+  for (int gi = 0; gi < ng; ++gi) dL_dalpha[gi] = ab[gi] / unit;
   if (st_bits & (ST_TIMEOUT | ST_NONFINITE)) return sim->fail(CASIM_E_NONFINITE, "adjoint pass: device status");
   return CASIM_OK;
 }

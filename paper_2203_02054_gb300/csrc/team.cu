@@ -665,7 +665,13 @@ __device__ __forceinline__ int team_scalars(const DW (&t)[3], bool first, CgStat
   } else {
     cg.rr = t[2];
     if (t[2].hi <= (float)cg.thr) return CG_DONE;
-    alpha = dw_div_fast(dw_mul(t[0], cg.q), dw_add_sloppy(dw_mul(t[1], cg.q), dw_neg(dw_mul(t[0], t[0]))));
+    // gamma brought to [1, 2) by a power of two, and the others with it: their
+    // products, squares of squared residuals, would leave FP32's range for
+    // residuals below 1e-10 or above 1e9
+    const int e = min(max(((__float_as_int(t[0].hi) >> 23) & 255) - 127, -126), 126);
+    const float sc = __int_as_float((127 - e) << 23);
+    const DW g{t[0].hi * sc, t[0].lo * sc}, dl{t[1].hi * sc, t[1].lo * sc}, q{cg.q.hi * sc, cg.q.lo * sc};
+    alpha = dw_div_fast(dw_mul(g, q), dw_add_sloppy(dw_mul(dl, q), dw_neg(dw_mul(g, g))));
     tb = dw_div_fast(t[0], cg.gamma).hi;
   }
   ta = alpha.hi;

@@ -93,3 +93,21 @@ def test_coarse_correction_cuts_the_iterations():
             its.append([h["pcg_iters"] for h in sim.history()])
             sim.close()
         assert its[0][0] < 0.5 * its[1][0] and its[0][3] < 0.6 * its[1][3], its
+
+
+@pytest.mark.parametrize("unit", [1e-7, 1e6])
+@pytest.mark.parametrize("shape", [(20, 4, 4, 4), (60, 11, 13, 8)])
+def test_mixed_in_other_units(shape, unit):
+    # squared residuals near FP32's range; one cluster and one team of blocks
+    m = _robot(*shape, seed=23, precision=MIXED)
+    X0 = _start(m, 4) * unit
+    X0 = X0.astype(np.float32).astype(np.float64)
+    m.rest = m.rest * unit
+    m.collision = synth.COLLISION_OFF
+    sim = casim.Sim(m)
+    sim.set_positions(X0)
+    sim.step(1)
+    assert sim.sync() == 0
+    X = sim.positions()
+    sim.close()
+    _check(m, X0, X)
