@@ -1483,10 +1483,8 @@ __device__ void spring_update_vertex(const Dev<T>& d, int qi, bool in_mesh, int 
   }
 }
 
-// Spring update of every query vertex, one thread each (the hash broad
-// phase's narrow phase runs one warp per vertex, which would leave 31 lanes
-// idle during this FP64 work; the tree's narrow phase runs one thread per
-// vertex and does the update in the same launch).
+// Spring update of every query vertex, one thread each, and the contact counts
+// of the narrow phase.
 template <typename T>
 __global__ void __launch_bounds__(128) k_springs(Dev<T> d) {
   __shared__ int shi[32];
