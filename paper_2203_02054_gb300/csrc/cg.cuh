@@ -241,8 +241,6 @@ __device__ __forceinline__ void finalize_iteration(const Dev<T>& d, double energ
   rec->energy = energy;
   if (!isfinite(energy) && d.stats) c->status |= ST_NONFINITE;
   c->iter += 1;
-  c->n_cast = 0;
-  if (d.tm_springs && d.n_robots == 1) d.tm_springs[0] = 0;
   for (int j = 0; j < 3; ++j) {
     c->box_lo[j] = 0x7FFFFFFFFFFFFFFFLL;
     c->box_hi[j] = (long long)0x8000000000000000ULL;

@@ -435,6 +435,18 @@ __device__ __forceinline__ bool may_be_inside_at(const R4<T>* X, const float (&p
   return may_be_inside(e[0], e[1], e[2], e[3], 0x1p-22f * dl);
 }
 
+// Zeroes the iteration's ray-cast list length and spring counts, which the spring
+// update counts up and the casts and the solve read; by the threads of the first
+// launch of the contact check, so whatever an iteration that ended early (a solve
+// that gave up, a launch that failed) left there is gone.
+template <typename T>
+__device__ __forceinline__ void start_counts(const Dev<T>& d) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t == 0) d.ctrl->n_cast = 0;
+  if (d.tm_springs)
+    for (int r = t; r < d.n_robots; r += gridDim.x * blockDim.x) d.tm_springs[r] = 0;
+}
+
 static constexpr int BRICK = 3;  // edge of the bricks of cells that k_tets looks up at once
 
 // Empty slot of a pair list (above every tet id).
@@ -466,6 +478,7 @@ template <typename T>
 __global__ void __launch_bounds__(QUERY_THREADS, 4) k_queries(Dev<T> d) {
   __shared__ int shi[32];
   const int qi = blockIdx.x * QUERY_THREADS + threadIdx.x;
+  start_counts(d);
   int n_obs = 0;
   if (qi < d.n_q) {
     const int v = d.q_verts[qi];
@@ -829,6 +842,7 @@ __global__ void __launch_bounds__(NARROW_BVH_THREADS, 4) k_narrow_bvh(Dev<T> d) 
   const int qi = (blockIdx.x * NARROW_BVH_THREADS + threadIdx.x) / TEAM_LANES;
   const int tl = threadIdx.x & (TEAM_LANES - 1);
   TeamStack& stack = s_stack[threadIdx.x / TEAM_LANES];
+  start_counts(d);
   int n_obs = 0;
   const bool valid = qi < d.n_q;
   const int v = valid ? d.q_verts[qi] : 0;
@@ -1426,7 +1440,7 @@ __device__ void spring_update_vertex(const Dev<T>& d, int qi, bool in_mesh, int 
     } else if (d.pair_count[qi] > 0) {
       deferred = true;
       const int slot = atomicAdd(&d.ctrl->n_cast, 1);  // < n_q: each vertex enters once
-      d.cast_list[slot] = qi;
+      if (slot < d.n_q) d.cast_list[slot] = qi;
     } else if (active) {
       if (kind == 1) {
         const V3 c = {d.spheres[4 * face], d.spheres[4 * face + 1], d.spheres[4 * face + 2]};
@@ -1642,7 +1656,7 @@ __global__ void __launch_bounds__(CAST_THREADS) k_cast(Dev<T> d) {
   const int lane = threadIdx.x & 31, tl = lane & 7;
   const unsigned tmask = 0xFFu << (lane & 24);
   const int n_warps = gridDim.x * (CAST_THREADS / 32);
-  const int n_cast = d.ctrl->n_cast;
+  const int n_cast = min(d.ctrl->n_cast, d.n_q);
   int active_out = 0;
   for (int j0 = 4 * (int)((blockIdx.x * (unsigned)CAST_THREADS + threadIdx.x) >> 5); j0 < n_cast; j0 += 4 * n_warps) {
     const int j = j0 + (lane >> 3);
@@ -1815,7 +1829,7 @@ __global__ void __launch_bounds__(NARROW_BVH_THREADS, 3) k_cast_bvh(Dev<T> d) {
   const int lane = threadIdx.x & 31, tl = lane & (TEAM_LANES - 1);
   TeamStack& stack = s_stack[threadIdx.x / TEAM_LANES];
   const int n_warps = gridDim.x * (NARROW_BVH_THREADS / 32);
-  const int n_cast = d.ctrl->n_cast;
+  const int n_cast = min(d.ctrl->n_cast, d.n_q);
   const BvhDev& b = d.bf;
   int active_out = 0;
   for (int j0 = 4 * (int)((blockIdx.x * (unsigned)NARROW_BVH_THREADS + threadIdx.x) >> 5); j0 < n_cast;

@@ -74,7 +74,7 @@ struct Ctrl {
   unsigned queue;        // next robot for the cluster PCG work queue
   long long iter;        // outer iterations completed (history index)
   long long total_pcg;   // PCG iterations summed over outer iterations
-  int n_cast;            // ray-cast list length of this iteration (reset at its end)
+  int n_cast;            // ray-cast list length of this iteration (reset by its contact check)
   long long box_lo[3];   // bounding box of all item boxes of this iteration,
   long long box_hi[3];   //   as order-preserving integer codes of doubles
 };

@@ -1403,8 +1403,6 @@ __global__ void k_finalize(Dev<T> d) {
   double at = 0.0;
 #pragma unroll
   for (int k = 0; k < K; ++k) at += a[k];
-  if (d.tm_springs && d.n_robots > 1)
-    for (int r = threadIdx.x; r < d.n_robots; r += blockDim.x) d.tm_springs[r] = 0;
   const double t = block_sum(at, sh);
   if (threadIdx.x == 0) finalize_iteration(d, t);
 }

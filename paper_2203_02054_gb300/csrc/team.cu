@@ -843,6 +843,7 @@ __global__ void __launch_bounds__(NTMAX, 1) k_pcg_team(const __grid_constant__ D
     T ta = T(0), tb = T(0);
     float gs = 0.0f, gr = 0.0f;  // lane l < 12 of every warp: g(s) and g(r)
     int it = -1, f = CG_CONTINUE;
+    bool lost = false;  // a wait gave up
     for (;; ++it) {
       const unsigned e = (unsigned)it + 2u;  // epoch of this pass's u and round
       A a[3];
@@ -1056,7 +1057,8 @@ __global__ void __launch_bounds__(NTMAX, 1) k_pcg_team(const __grid_constant__ D
         cluster_wait();
       } else {
         __syncthreads();
-        if (!s_ok) return;
+        lost = !s_ok;
+        if (lost) break;
       }
       {
         // The team's totals and the shares of g(w) and g(r).  FP32: warp 0
@@ -1140,7 +1142,10 @@ __global__ void __launch_bounds__(NTMAX, 1) k_pcg_team(const __grid_constant__ D
           }
         }
         __syncthreads();
-        if (!CL && s_lost) return;
+        if constexpr (!CL) {
+          lost = s_lost;
+          if (lost) break;
+        }
         ta = s_ta;
         tb = s_tb;
         f = s_flag;
@@ -1179,6 +1184,12 @@ __global__ void __launch_bounds__(NTMAX, 1) k_pcg_team(const __grid_constant__ D
             s[q][k] = w[q][k] + tb * s[q][k];
           }
       }
+    }
+    if (lost) {
+      // the positions stay as they are; the iteration's record is closed all the
+      // same (a batch's by the finalize launch)
+      if (d.n_robots == 1 && d.rhs_in_pcg && c.me == 0 && t == 0) finalize_iteration(d, 0.0);
+      return;
     }
     it = max(it, 0);
     if (it > 0) {
