@@ -1467,11 +1467,12 @@ static cudaLaunchConfig_t team_config(int grid, int threads, size_t smem, bool c
 }
 
 // Raises the kernel's shared-memory limit (and allows its cluster size); false
-// when it cannot be resident.
+// when it cannot be resident.  The limit belongs to the kernel and every handle's
+// launches share it: always the same, so that no upload lowers another's.
 bool team_prepare(bool fp64, int r, bool cluster, int grid, int threads, size_t smem) {
   const bool ok = with_team_kernel(fp64, r, cluster, [&](auto k) {
     int n = 0;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return false;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TEAM_SMEM_MAX) != cudaSuccess) return false;
     if (!cluster)
       return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem) == cudaSuccess && n >= 1;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
