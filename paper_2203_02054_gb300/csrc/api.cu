@@ -726,7 +726,8 @@ int upload_team(casim_sim* sim) {
     // one matrix per level and robot: A_c + sigma I; scratch of the inversion:
     // matrices, panels, pivots, offsets, dimensions, flags
     const int n = TEAM_LEVELS * nm;
-    const size_t nl = h.Ac.size(), nA = TEAM_LEVELS * nl, nC = (size_t)n * mx * 32, nD = (size_t)n * 32 * 32;
+    const size_t ns = std::min(n, INVERT_SLICE);
+    const size_t nl = h.Ac.size(), nA = TEAM_LEVELS * nl, nC = ns * mx * 32, nD = ns * 32 * 32;
     char* tmp = nullptr;
     const size_t bytes = sizeof(double) * (nA + nC + nD) + sizeof(long long) * n + 2 * sizeof(int) * (size_t)n;
     CK(cudaMalloc(&tmp, bytes));

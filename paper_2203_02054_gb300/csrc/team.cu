@@ -1373,23 +1373,37 @@ __global__ void k_shift(double* A, const long long* off, const int* dim, double 
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i < n) A[off[blockIdx.y] + i * (n + 1)] += sigma;
 }
+
+// Calls f(first, count) for n_mat matrices (a batch has TEAM_LEVELS a robot) in
+// slices that fit a grid's y and z dimensions.
+template <typename F>
+static void for_slices(int n_mat, F f) {
+  for (int s = 0; s < n_mat; s += INVERT_SLICE) f(s, std::min(INVERT_SLICE, n_mat - s));
+}
+
 void launch_shift(double* A, const long long* off, const int* dim, int n_mat, double sigma, cudaStream_t st) {
-  k_shift<<<dim3((4 * TEAM_MAX_PARTS + 255) / 256, n_mat), 256, 0, st>>>(A, off, dim, sigma);
+  for_slices(n_mat, [&](int s, int m) {
+    k_shift<<<dim3((4 * TEAM_MAX_PARTS + 255) / 256, m), 256, 0, st>>>(A, off + s, dim + s, sigma);
+  });
 }
 
 // Inverts n_mat matrices at A + off[r] (dim[r] rows, at most max_dim) into out
-// (same offsets).  C holds n_mat x max_dim x 32 doubles, D n_mat x 32 x 32;
+// (same offsets).  C holds m x max_dim x 32 doubles, D m x 32 x 32 for m matrices,
+// n_mat or INVERT_SLICE if that is less;
 // bad[r] becomes 1 for a matrix that is not positive definite.
 void launch_invert(double* A, const long long* off, const int* dim, int n_mat, int max_dim, double* C, double* D,
                    float* out, int* bad, cudaStream_t st) {
-  const int nk = (max_dim + GJ - 1) / GJ;
-  for (int kb = 0; kb < nk; ++kb) {
-    k_gj_pivot<<<n_mat, dim3(GJ, GJ), 0, st>>>(A, off, dim, kb, D, bad);
-    k_gj_row<<<dim3(nk, n_mat), dim3(GJ, GJ), 0, st>>>(A, off, dim, kb, D, C, max_dim);
-    const int nt = (max_dim + 2 * GJ - 1) / (2 * GJ);
-    k_gj_update<<<dim3(nt, nt, n_mat), 256, 0, st>>>(A, off, dim, kb, D, C, max_dim);
-  }
-  k_gj_float<<<dim3(std::min(((max_dim * max_dim) + 255) / 256, 1024), n_mat), 256, 0, st>>>(A, off, dim, out, bad);
+  const int nk = (max_dim + GJ - 1) / GJ, nt = (max_dim + 2 * GJ - 1) / (2 * GJ);
+  for_slices(n_mat, [&](int s, int m) {
+    const long long* o = off + s;
+    const int* n = dim + s;
+    for (int kb = 0; kb < nk; ++kb) {
+      k_gj_pivot<<<m, dim3(GJ, GJ), 0, st>>>(A, o, n, kb, D, bad + s);
+      k_gj_row<<<dim3(nk, m), dim3(GJ, GJ), 0, st>>>(A, o, n, kb, D, C, max_dim);
+      k_gj_update<<<dim3(nt, nt, m), 256, 0, st>>>(A, o, n, kb, D, C, max_dim);
+    }
+    k_gj_float<<<dim3(std::min(((max_dim * max_dim) + 255) / 256, 1024), m), 256, 0, st>>>(A, o, n, out, bad + s);
+  });
 }
 
 // ---------------------------------------------------------------- launchers

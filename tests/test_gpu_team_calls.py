@@ -1,12 +1,21 @@
-"""Calls around the team PCG: several handles in one process."""
+"""Calls around the team PCG: several handles in one process, and batches of very many
+robots."""
 import numpy as np
 import pytest
 
 from paper_2203_02054_gb300 import casim, synth
+from oracle import loop, springs as osprings
 
 pytestmark = pytest.mark.gpu
 
 FP64, MIXED = synth.PRECISION_FP64, synth.PRECISION_MIXED
+BAR = {FP64: 1e-9, MIXED: 1e-5}
+
+
+def _want(m, X0, collision):
+    prep = loop.prepare(m.rest, m.tets, m.group, m.fixed)
+    return loop.iterate(prep, X0, osprings.SpringState.empty(prep.query.shape[0]), m.alpha, m.spheres, m.w_knots,
+                        m.k_spring, m.eps, collision)[0]
 
 
 def _fingers(precision, sizes):
@@ -40,3 +49,25 @@ def test_an_upload_leaves_other_handles_alone(precision, first, second):
             s.close()
     for X in runs[1:]:
         assert np.array_equal(X, runs[0])
+
+
+def test_batch_of_very_many_robots():
+    n = 11000
+    rest, tets, group, fixed = synth._voxel_kuhn(1, 1, 2, 0.5, group_of_voxel=lambda i, j, k: 0)
+    m = synth.config1_beam()
+    m.rest, m.tets, m.group, m.fixed = rest, tets, group, fixed
+    m.precision, m.collision = MIXED, synth.COLLISION_OFF
+    robots = []
+    for r in range(n):
+        q = synth.Mesh(**vars(m)) if r else m
+        q.alpha = np.array([1.1 + 0.5 * r / n])
+        robots.append(q)
+    sim = casim.Sim(robots)
+    assert sim.stats().pcg_kernel == 5
+    sim.step(1)
+    assert sim.sync() == 0
+    X = sim.positions().reshape(n, m.n_verts, 3)
+    sim.close()
+    for r in (0, 1, n // 2, n - 1):
+        want = _want(robots[r], m.rest, 0)
+        assert np.abs(X[r] - want).max() <= BAR[MIXED] * m.bbox_diag()
