@@ -228,10 +228,11 @@ struct TeamHost {
   size_t smem = 0;
   int ainv_off = 0, val_off = 0, lcol_off = 0;
   // length of a robot's parts: as few parts as possible, equally long (a
-  // round takes as long as the longest), in whole warps
+  // round takes as long as the longest), in whole warps; at least one, also for a
+  // robot without free rows, which has no part
   int part_rows(int robot_rows) const {
     const int np = std::max(1, (robot_rows + rows - 1) / rows);
-    return ((robot_rows + np - 1) / np + 31) & ~31;
+    return std::max(32, ((robot_rows + np - 1) / np + 31) & ~31);
   }
 };
 struct TeamDevice {

@@ -1,5 +1,5 @@
-"""Calls around the team PCG: several handles in one process, and batches of very many
-robots."""
+"""Calls around the team PCG: several handles in one process, batches of very many
+robots, and robots without a free vertex."""
 import numpy as np
 import pytest
 
@@ -71,3 +71,24 @@ def test_batch_of_very_many_robots():
     for r in (0, 1, n // 2, n - 1):
         want = _want(robots[r], m.rest, 0)
         assert np.abs(X[r] - want).max() <= BAR[MIXED] * m.bbox_diag()
+
+
+@pytest.mark.parametrize("precision", [FP64, MIXED])
+@pytest.mark.parametrize("at", [0, 1, 2])
+def test_a_robot_without_free_vertices(precision, at):
+    ms = _fingers(precision, [(20, 4, 4, 4), (12, 4, 4, 2), (23, 5, 5, 3)])
+    ms[at].fixed = np.ones_like(ms[at].fixed)
+    dtype = np.float64 if precision == FP64 else np.float32
+    X0 = [m.rest.copy() if k == at else synth.perturbed_positions(m, 0.25, seed=60 + k, dtype=dtype)
+          for k, m in enumerate(ms)]
+    sim = casim.Sim(ms)
+    assert sim.stats().pcg_kernel == 5
+    sim.set_positions(np.concatenate(X0))
+    sim.step(1)
+    assert sim.sync() == 0
+    X = sim.positions()
+    sim.close()
+    o = np.cumsum([0] + [m.n_verts for m in ms])
+    for k, m in enumerate(ms):
+        want = X0[k] if k == at else _want(m, X0[k], m.collision)
+        assert np.abs(X[o[k]:o[k + 1]] - want).max() <= BAR[precision] * m.bbox_diag()
