@@ -1192,12 +1192,13 @@ __global__ void __launch_bounds__(NTMAX, 1) k_pcg_team(const __grid_constant__ D
       return;
     }
     it = max(it, 0);
-    if (it > 0) {
+    if (it > 0 || d.xstep) {
 #pragma unroll
       for (int q = 0; q < R; ++q)
         if (act[q]) {
-          // x_(i+1) = start + correction; the step x_(i+1) - x_i is kept for
-          // the next outer iteration's start
+          // x_(i+1) = start + correction (zero if the start already meets the
+          // tolerance: that is where its residual was formed); the step x_(i+1) -
+          // x_i is kept for the next outer iteration's start
           const int i = row0 + lt + q * rt;
           if constexpr (F32) {
             const R4<T> x0 = d.X[i];

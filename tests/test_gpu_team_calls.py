@@ -1,10 +1,10 @@
 """Calls around the team PCG: several handles in one process, batches of very many
-robots, and robots without a free vertex."""
+robots, robots without a free vertex, and solves that need no iteration."""
 import numpy as np
 import pytest
 
 from paper_2203_02054_gb300 import casim, synth
-from oracle import loop, springs as osprings
+from oracle import global_step, local, loop, springs as osprings
 
 pytestmark = pytest.mark.gpu
 
@@ -92,3 +92,44 @@ def test_a_robot_without_free_vertices(precision, at):
     for k, m in enumerate(ms):
         want = X0[k] if k == at else _want(m, X0[k], m.collision)
         assert np.abs(X[o[k]:o[k + 1]] - want).max() <= BAR[precision] * m.bbox_diag()
+
+
+@pytest.mark.parametrize("n_robots", [1, 3])
+def test_a_solve_without_iterations_returns_where_its_residual_was_tested(n_robots):
+    """With a loose tolerance the extrapolated start soon meets it.  The positions
+    returned then have a residual within the tolerance, the ones the iteration
+    came from had not (several times above it along this trajectory)."""
+    tol = 5e-5
+    ms = [synth.small_finger(20, 4, 4, 4, seed=7 + r, n_iters=30) for r in range(n_robots)]
+    for m in ms:
+        m.collision = synth.COLLISION_OFF
+    preps = [loop.prepare(m.rest, m.tets, m.group, m.fixed) for m in ms]
+    o = np.cumsum([0] + [m.n_verts for m in ms])
+
+    def residual(k, Xi, X):
+        """of the global step of robot k that starts from Xi, at X"""
+        m, p = ms[k], preps[k]
+        P = local.local_step(Xi, p.tets, p.T_c, p.vol0, p.group, m.alpha, m.w_knots)[0]
+        A, b = global_step.assemble(p.tets, p.omega, P, p.n_verts, [], np.zeros((0, 3)), m.k_spring)
+        free = ~p.fixed.astype(bool)
+        rhs = b[free] - A[free][:, ~free] @ X[~free]
+        return np.linalg.norm(rhs - A[free][:, free] @ X[free]) / np.linalg.norm(rhs)
+
+    sim = casim.Sim(ms if n_robots > 1 else ms[0], pcg_tol=tol)
+    assert sim.stats().pcg_kernel == 5
+    X = np.concatenate([m.rest for m in ms])
+    none = 0
+    for _ in range(30):
+        Xi = X.astype(np.float64)
+        sim.step(1)
+        assert sim.sync() == 0
+        X = sim.positions().astype(np.float64)
+        if sim.history()[-1]["pcg_iters"] == 0:
+            none += 1
+            for k in range(n_robots):
+                s = slice(o[k], o[k + 1])
+                assert residual(k, Xi[s], Xi[s]) > tol
+                # (5 %: FP32 targets are within 1e-6 of the right-hand side)
+                assert residual(k, Xi[s], X[s]) <= 1.05 * tol
+    sim.close()
+    assert none > 0  # (premise: such solves occurred)
