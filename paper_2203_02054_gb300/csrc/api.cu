@@ -225,6 +225,7 @@ struct TeamHost {
   int halo_max = 0, max_np = 0;
   bool coarse = false;
   bool constants = false;  // coarse basis of constants alone, without sigma
+  int levels = TEAM_LEVELS;  // inverses: one where no solve takes another (no springs, no sigma)
   size_t smem = 0;
   int ainv_off = 0, val_off = 0, lcol_off = 0;
   // length of a robot's parts: as few parts as possible, equally long (a
@@ -482,7 +483,7 @@ Dev<T> make_dev(casim_sim* sim) {
   d.tm_lcol_off = sim->team.lcol_off;
   d.tm_cluster = sim->team.cluster;
   d.tm_coarse = sim->team.coarse ? 1 : 0;
-  d.tm_levels = sim->team.constants ? 1 : TEAM_LEVELS;
+  d.tm_levels = sim->team.levels;
   d.tm_halo_max = sim->team.halo_max;
   d.tm_halo = sim->tm.halo;
   d.tm_lcol = sim->tm.lcol;
@@ -726,9 +727,9 @@ int upload_team(casim_sim* sim) {
     CK(up(g.z, h.z.data(), sizeof(float4) * h.z.size()));
     // one matrix per level and robot: A_c + sigma I; scratch of the inversion:
     // matrices, panels, pivots, offsets, dimensions, flags
-    const int n = TEAM_LEVELS * nm;
+    const int nlev = h.levels, n = nlev * nm;
     const size_t ns = std::min(n, INVERT_SLICE);
-    const size_t nl = h.Ac.size(), nA = TEAM_LEVELS * nl, nC = ns * mx * 32, nD = ns * 32 * 32;
+    const size_t nl = h.Ac.size(), nA = nlev * nl, nC = ns * mx * 32, nD = ns * 32 * 32;
     char* tmp = nullptr;
     const size_t bytes = sizeof(double) * (nA + nC + nD) + sizeof(long long) * n + 2 * sizeof(int) * (size_t)n;
     CK(cudaMalloc(&tmp, bytes));
@@ -738,8 +739,8 @@ int upload_team(casim_sim* sim) {
     int *dim = reinterpret_cast<int*>(off + n), *bad = dim + n;
     std::vector<int> bad_h(n, 0), dim_h;
     std::vector<long long> off_h;
-    std::vector<double> shift(TEAM_LEVELS, 0.0);
-    for (int l = 0; l < TEAM_LEVELS; ++l) {
+    std::vector<double> shift(nlev, 0.0);
+    for (int l = 0; l < nlev; ++l) {
       if (l) shift[l] = sim->params.k_spring * TEAM_SIGMA_1 * std::pow(4.0, l - 1);
       for (int r = 0; r < nm; ++r) {
         off_h.push_back(h.ac_off[r] + (long long)(l * nl));
@@ -747,13 +748,13 @@ int upload_team(casim_sim* sim) {
       }
     }
     cudaError_t e = up(A, h.Ac.data(), sizeof(double) * nl);
-    for (int l = 1; l < TEAM_LEVELS && e == cudaSuccess; ++l)
+    for (int l = 1; l < nlev && e == cudaSuccess; ++l)
       e = cudaMemcpyAsync(A + l * nl, A, sizeof(double) * nl, cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess) e = up(off, off_h.data(), sizeof(long long) * n);
     if (e == cudaSuccess) e = up(dim, dim_h.data(), sizeof(int) * n);
     if (e == cudaSuccess) e = cudaMemsetAsync(bad, 0, sizeof(int) * n, st);
     if (e == cudaSuccess) {
-      for (int l = 1; l < TEAM_LEVELS; ++l) launch_shift(A, off + l * nm, dim + l * nm, nm, shift[l], st);
+      for (int l = 1; l < nlev; ++l) launch_shift(A, off + l * nm, dim + l * nm, nm, shift[l], st);
       launch_invert(A, off, dim, n, mx, C, D, g.ainv, bad, st);
       e = cudaGetLastError();
     }
@@ -835,7 +836,7 @@ int upload_typed(casim_sim* sim, const std::vector<double>& rest_int, const std:
     g.r = sim->dalloc<R4<double>>(n_free);
     if (h.coarse) {
       g.z = sim->dalloc<float4>(n_free);
-      g.ainv = sim->dalloc<float>(TEAM_LEVELS * h.Ac.size());
+      g.ainv = sim->dalloc<float>(h.levels * h.Ac.size());
       g.ainv_level = h.Ac.size();
     }
     g.springs = sim->dalloc<int>(sim->n_robots);
@@ -1639,6 +1640,7 @@ void build_team(casim_sim* sim, const std::vector<double>& rest_int,
   // where a twelfth of the runs go (7 of 80 over ten iterations); with this
   // basis they follow the trajectories they always did.
   h.constants = !fp64 && sim->n_robots == 1 && n_free <= TEAM_CONSTANTS_MAX;
+  h.levels = h.constants || sim->params.collision == 0 ? 1 : TEAM_LEVELS;
   if (h.coarse) {
     // basis of every part: 1 and the rest coordinates, orthonormalised in that
     // order; a function that depends on the earlier ones (a part with fewer
