@@ -235,6 +235,8 @@ struct TeamHost {
     const int np = std::max(1, (robot_rows + rows - 1) / rows);
     return std::max(32, ((robot_rows + np - 1) / np + 31) & ~31);
   }
+  int pieces = 1;  // constants: pieces of 96 rows of a part, each with a constant of its own
+  int leaf_rows(int robot_rows) const { return part_rows(robot_rows) / pieces; }
 };
 struct TeamDevice {
   TeamPart* part = nullptr;
@@ -1559,10 +1561,28 @@ void plan_team(const casim_params& p, const std::vector<int>& rows, TeamHost& h)
     take(3, TEAM_NT_F64);
     return;
   }
+  // Small single robots in MIXED keep the constants alone over 96 rows, without
+  // sigma: their runs are decided by single contacts (one decision that falls
+  // the other way moves a 570-vertex finger by 5e-5 of its size), so a solve
+  // that leaves another error of the same size within the tolerance changes
+  // where a twelfth of the runs go (7 of 80 over ten iterations; 3 of 80 at 1,536
+  // to 4,096 rows); with this basis they follow the trajectories they always did.
+  h.constants = rows.size() == 1 && biggest <= TEAM_CONSTANTS_MAX;
   if (p.pcg_block) {
     take(1, p.pcg_block);
     return;
   }
+  // Beyond one cluster of 96-row parts, the constants of two or three pieces of
+  // 96 rows go into one part, so that the team still is a cluster: 187, 206 and
+  // 241 us per solve at 1,953, 3,132 and 3,852 rows (43 to 47 iterations); 222, 241
+  // and 263 us with 96-row parts, whose rounds go through L2.
+  if (h.constants && biggest > 96 * TEAM_CLUSTER)
+    for (int n = 2; n <= 3; ++n)
+      if (parts(96 * n) <= TEAM_CLUSTER) {
+        h.pieces = n;
+        take(1, 96 * n);
+        return;
+      }
   for (int len = 96; len <= TEAM_NT_1; len += 32)
     if (parts(len) <= sms) {
       take(1, len);
@@ -1633,20 +1653,15 @@ void build_team(casim_sim* sim, const std::vector<double>& rest_int,
   }
   if (h.halo.empty()) h.halo.push_back(0);
   h.coarse = sim->params.pcg_precond == 0;
-  // Small single robots in MIXED keep the constants alone over 96 rows, without
-  // sigma: their runs are decided by single contacts (one decision that falls
-  // the other way moves a 570-vertex finger by 5e-5 of its size), so a solve
-  // that leaves another error of the same size within the tolerance changes
-  // where a twelfth of the runs go (7 of 80 over ten iterations); with this
-  // basis they follow the trajectories they always did.
-  h.constants = !fp64 && sim->n_robots == 1 && n_free <= TEAM_CONSTANTS_MAX;
   h.levels = h.constants || sim->params.collision == 0 ? 1 : TEAM_LEVELS;
   if (h.coarse) {
     // basis of every part: 1 and the rest coordinates, orthonormalised in that
     // order; a function that depends on the earlier ones (a part with fewer
-    // than four rows, or a flat one) becomes zero, its diagonal entry one
+    // than four rows, or a flat one) becomes zero, its diagonal entry one.
+    // With constants alone: 1 on each piece of the part
     h.z.assign(std::max(n_free, 1), make_float4(0.0f, 0.0f, 0.0f, 0.0f));
     std::vector<double> q;
+    const int piece = h.leaf_rows(n_free);
     std::vector<char> dead(4 * h.part.size(), 0);
     for (size_t p = 0; p < h.part.size(); ++p) {
       const int r0 = h.part[p].row0, m = h.part[p].nrow;
@@ -1655,7 +1670,9 @@ void build_team(casim_sim* sim, const std::vector<double>& rest_int,
         double* v = q.data() + (size_t)f * m;
         double size = 0.0, left = 0.0;
         for (int i = 0; i < m; ++i) {
-          v[i] = f == 0 ? 1.0 : rest_int[3 * (size_t)(r0 + i) + f - 1] - rest_int[3 * (size_t)r0 + f - 1];
+          v[i] = h.constants ? (i / piece == f ? 1.0 : 0.0)
+                 : f == 0    ? 1.0
+                             : rest_int[3 * (size_t)(r0 + i) + f - 1] - rest_int[3 * (size_t)r0 + f - 1];
           size += v[i] * v[i];
         }
         for (int pass = 0; pass < 2; ++pass)
@@ -1666,7 +1683,7 @@ void build_team(casim_sim* sim, const std::vector<double>& rest_int,
             for (int i = 0; i < m; ++i) v[i] -= c * w[i];
           }
         for (int i = 0; i < m; ++i) left += v[i] * v[i];
-        const bool ok = left > 1e-12 * size && left > 0.0 && !(h.constants && f > 0);
+        const bool ok = left > 1e-12 * size && left > 0.0;
         const double s = ok ? 1.0 / std::sqrt(left) : 0.0;
         for (int i = 0; i < m; ++i) {
           v[i] *= s;
@@ -1849,7 +1866,7 @@ static int upload_robots(casim_sim* sim, int32_t n_verts, const double* rest_xyz
       if (!fixed[v]) per_robot[std::max(0, robot_of_vert_user[v])].push_back(v);
     for (int r = 0; r < n_robots; ++r) {
       std::vector<int>& L = per_robot[r];
-      rcb_order(rest_xyz, L.data(), (int)L.size(), parts ? sim->team.part_rows((int)L.size()) : 128);
+      rcb_order(rest_xyz, L.data(), (int)L.size(), parts ? sim->team.leaf_rows((int)L.size()) : 128);
       for (int v : L) sim->int_of_user[v] = nf++;
     }
   }

@@ -32,7 +32,7 @@ static constexpr int TEAM_NT_3 = 512;       //   three FP32 rows per thread,
 static constexpr int TEAM_NT_F64 = 384;     //   one FP64 column of up to three rows per thread
 static constexpr int TEAM_LEVELS = 6;        //   inverses of the coarse matrix: for no springs,
 static constexpr float TEAM_SIGMA_1 = 1.0f / 1024;  //   springs per row of the next one (then a factor 4 each)
-static constexpr int TEAM_CONSTANTS_MAX = 4096; //   MIXED robots up to this many rows: constant basis functions alone
+static constexpr int TEAM_CONSTANTS_MAX = 4096; //   single MIXED robots up to this many rows: constants alone (see plan_team)
 static constexpr int INVERT_SLICE = 16384;  //   matrices inverted at once (a grid's z has at most 65,535)
 static constexpr size_t TEAM_SMEM_MAX = 216 * 1024;  //   dynamic shared memory
 static constexpr int PCG_CL_SIZE = 16;   // CTAs per cluster (non-portable size)
