@@ -77,7 +77,8 @@ typedef struct {
   int32_t collision;        /* CASIM_COLLISION_*                                      */
   double k_spring;          /* spring weight k of Eq. 5 (Eq. 8 uses 1)                */
   double eps;               /* contact offset epsilon of Sec. II-C (length units)     */
-  double pcg_tol;           /* stop when |r|_2 <= pcg_tol * |b|_2                     */
+  double pcg_tol;           /* stop when |r|_2 <= pcg_tol * |b|_2 (kernel 5 in FP64
+                               with its two-level preconditioner: at 1/32 of it)      */
   int32_t pcg_max_iter;     /* PCG iteration cap per outer iteration                  */
   int32_t n_w_knots;        /* number of (strain, w) knots of R_omega, >= 1           */
   const double* w_knots;    /* host, 2*n_w_knots doubles (eps_i, w_i), eps ascending;
@@ -136,7 +137,9 @@ typedef struct {
                                energy statistic; the autotuner picks them        */
   int32_t pcg_block;        /* free vertices per block of the team PCG (5) in MIXED:
                                0 auto (the shortest blocks that one wave of the
-                               SMs holds, at least 96); 288 or 384 forces it      */
+                               SMs holds, at least 96; single robots of up to 4,096
+                               free vertices: 96, 192 or 288, the shortest with at
+                               most 16 blocks); 288 or 384 forces it              */
 } casim_params;
 
 #define CASIM_DEBUG_BARRIER_NEVER_COMPLETES 1

@@ -8,7 +8,7 @@ dimensions are
 * the global-step kernel and its preconditioner (``pcg_kernel``,
   ``pcg_precond``: for one robot the team kernel with the two-level or the
   Jacobi preconditioner, the register-resident and the streaming kernels; for
-  a batch the segmented and the cluster kernels) and the team kernel's
+  a batch the team and the cluster kernels) and the team kernel's
   rows per block (``pcg_block``),
 * the collision broad phase (``broad_phase``: spatial hash or AABB trees) and
   the hash cell edge (``cell_scale`` times the voxel edge),

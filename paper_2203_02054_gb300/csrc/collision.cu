@@ -314,10 +314,6 @@ __device__ __forceinline__ bool strictly_inside_at(const R4<T>* X, T px, T py, T
   if (orient_t(a.x, a.y, a.z, b.x, b.y, b.z, c.x, c.y, c.z, px, py, pz) <= 0) return false;
   return true;
 }
-template <typename T>
-__device__ __forceinline__ bool strictly_inside(const Dev<T>& d, T px, T py, T pz, int4 t) {
-  return strictly_inside_at(d.X, px, py, pz, t);
-}
 // The same behind a call: where it is rare, its registers stay out of the caller.
 template <typename T>
 __device__ __noinline__ bool strictly_inside_call(const R4<T>* X, T px, T py, T pz, int4 t) {
@@ -375,9 +371,6 @@ __device__ __forceinline__ void obstacle_tests(const Dev<T>& d, T px, T py, T pz
       if (strictly_inside_call(d.OX, px, py, pz, d.ot.prim[e])) ++n_mesh;
     });
 }
-
-template <typename T>
-__device__ void spring_update_vertex(const Dev<T>& d, int qi, int& active_out, unsigned long long& ssig);
 
 // Block totals of one spring-update launch into this iteration's record: self
 // pairs, finished springs and the springs' signature.
@@ -692,7 +685,7 @@ __global__ void __launch_bounds__(TETS_MAX_THREADS, 4) k_tets(Dev<T> d, int per_
         const int2 pr = s_pairs[wid][n_pairs - 1 - lane];
         const int v = d.q_verts[pr.y];
         if (!d.robot_of_tet || d.robot_of_vert[v] == d.robot_of_tet[pr.x]) {
-          // (strictly_inside, with the four signs in a loop around one inlined
+          // (strictly_inside_at, with the four signs in a loop around one inlined
           // copy of the exact arithmetic: a call would cost the walk its registers)
           const R4<T> x = d.X[v];
           const int4 pt = d.tet[pr.x];

@@ -160,6 +160,5 @@ int rhs_blocks(int n_free);
 int local_blocks(int n_t, int threads);
 int rhs_blocks(int n_free, int threads);
 int scan_tiles(int n);
-// ints to allocate after an (n + 1)-int count array for the single-pass scan
 
 }  // namespace casim

@@ -28,7 +28,8 @@
 // Preconditioner: M^-1 = D^-1 + Z (A_c + sigma I)^-1 Z^T, Jacobi plus an
 // additive coarse correction.  Z holds, for every part (a compact piece of the
 // body), the constant and the three linear functions of the rest position,
-// orthonormalised over the part; A_c = Z^T L Z is the Galerkin matrix of the
+// orthonormalised over the part (small MIXED robots: the constants of up to three
+// pieces of it, without sigma); A_c = Z^T L Z is the Galerkin matrix of the
 // spring-free Laplacian.  The springs add k Z^T diag(mask) Z to it, a
 // different block-diagonal matrix every iteration; sigma = k (springs / rows)
 // stands for it.  (Without it the coarse correction takes the body's soft
@@ -1247,7 +1248,8 @@ __global__ void __launch_bounds__(NTMAX, 1) k_pcg_team(const __grid_constant__ D
 // Gauss-Jordan elimination without pivoting: for every 32-wide pivot block,
 // its inverse D, the pivot rows D A_k*, the rank-32 update of all other rows,
 // and the pivot column -A_*k D.  On the device because the coarse matrix of a
-// large robot has up to 1,824 rows: 2 n^3 operations, seconds on the host.
+// large robot has up to 640 rows (4 TEAM_MAX_PARTS): 2 n^3 operations for each
+// robot and level.
 static constexpr int GJ = 32;
 
 __device__ __forceinline__ double* gj_mat(double* A, const long long* off, const int* dim, int r, int& n) {
