@@ -710,8 +710,28 @@ cudaError_t enqueue_iteration(casim_sim* sim, cudaStream_t st, cudaEvent_t* ev, 
   return cudaGetLastError();
 }
 
-// The team PCG's tables, and the inverses of its coarse matrices (on the
-// device; a matrix that is not positive definite leaves Jacobi alone).
+// Drops robot r's coarse functions f0 .. 3 of every part from the basis and from
+// its matrix (its diagonal entries become one).
+void drop_functions(TeamHost& h, int r, int f0) {
+  const long long nd = h.ac_dim[r];
+  double* Ac = h.Ac.data() + h.ac_off[r];
+  for (const TeamPart& t : h.part)
+    if (t.robot == r)
+      for (int i = t.row0; i < t.row0 + t.nrow; ++i)
+        for (int f = f0; f < 4; ++f) (&h.z[i].x)[f] = 0.0f;
+  for (long long i = 0; i < nd; ++i)
+    for (long long j = 0; j < nd; ++j)
+      if (i % 4 >= f0 || j % 4 >= f0) Ac[i * nd + j] = i == j ? 1.0 : 0.0;
+}
+
+// The team PCG's tables, and the inverses of its coarse matrices, formed on the
+// device and kept in FP32.  A robot whose matrix is too ill-conditioned for that
+// (the rounding of the inverse, relative to its smallest eigenvalue, is about
+// 2^-24 |A_c| |A_c^-1|) does without the linear functions, whose matrix has the
+// larger norm, and failing that without a correction.  Bodies of 300 x 2 x 2
+// voxels reach 0.02 with the linear functions, of 1,200 0.18, and of 1,500 0.28,
+// where FP64 solves no longer converged with them, nor MIXED ones at 1.0 (3,000
+// voxels); constants alone reach 0.03 at 4,000.
 int upload_team(casim_sim* sim) {
   TeamHost& h = sim->team;
   TeamDevice& g = sim->tm;
@@ -726,18 +746,20 @@ int upload_team(casim_sim* sim) {
   if (h.coarse) {
     const int nm = (int)h.ac_dim.size();
     const int mx = *std::max_element(h.ac_dim.begin(), h.ac_dim.end());
-    CK(up(g.z, h.z.data(), sizeof(float4) * h.z.size()));
     // one matrix per level and robot: A_c + sigma I; scratch of the inversion:
-    // matrices, panels, pivots, offsets, dimensions, flags
+    // matrices, panels, pivots, offsets, norms of A_c and its inverse, dimensions,
+    // flags
     const int nlev = h.levels, n = nlev * nm;
     const size_t ns = std::min(n, INVERT_SLICE);
     const size_t nl = h.Ac.size(), nA = nlev * nl, nC = ns * mx * 32, nD = ns * 32 * 32;
     char* tmp = nullptr;
-    const size_t bytes = sizeof(double) * (nA + nC + nD) + sizeof(long long) * n + 2 * sizeof(int) * (size_t)n;
+    const size_t bytes =
+        sizeof(double) * (nA + nC + nD + 2 * (size_t)nm) + sizeof(long long) * n + 2 * sizeof(int) * (size_t)n;
     CK(cudaMalloc(&tmp, bytes));
     double* A = reinterpret_cast<double*>(tmp);
     double *C = A + nA, *D = C + nC;
-    long long* off = reinterpret_cast<long long*>(D + nD);
+    double* norm = D + nD;
+    long long* off = reinterpret_cast<long long*>(norm + 2 * nm);
     int *dim = reinterpret_cast<int*>(off + n), *bad = dim + n;
     std::vector<int> bad_h(n, 0), dim_h;
     std::vector<long long> off_h;
@@ -749,24 +771,41 @@ int upload_team(casim_sim* sim) {
         dim_h.push_back(h.ac_dim[r]);
       }
     }
-    cudaError_t e = up(A, h.Ac.data(), sizeof(double) * nl);
-    for (int l = 1; l < nlev && e == cudaSuccess; ++l)
-      e = cudaMemcpyAsync(A + l * nl, A, sizeof(double) * nl, cudaMemcpyDeviceToDevice, st);
-    if (e == cudaSuccess) e = up(off, off_h.data(), sizeof(long long) * n);
+    std::vector<double> norm_h(2 * (size_t)nm);
+    std::vector<int> dropped(nm, 0);  // 1: the linear functions, 2: all
+    cudaError_t e = up(off, off_h.data(), sizeof(long long) * n);
     if (e == cudaSuccess) e = up(dim, dim_h.data(), sizeof(int) * n);
-    if (e == cudaSuccess) e = cudaMemsetAsync(bad, 0, sizeof(int) * n, st);
-    if (e == cudaSuccess) {
-      for (int l = 1; l < nlev; ++l) launch_shift(A, off + l * nm, dim + l * nm, nm, shift[l], st);
-      launch_invert(A, off, dim, n, mx, C, D, g.ainv, bad, st);
-      e = cudaGetLastError();
+    for (bool again = true; again && e == cudaSuccess;) {
+      again = false;
+      e = up(A, h.Ac.data(), sizeof(double) * nl);
+      for (int l = 1; l < nlev && e == cudaSuccess; ++l)
+        e = cudaMemcpyAsync(A + l * nl, A, sizeof(double) * nl, cudaMemcpyDeviceToDevice, st);
+      if (e == cudaSuccess) e = cudaMemsetAsync(bad, 0, sizeof(int) * n, st);
+      if (e == cudaSuccess) e = cudaMemsetAsync(norm, 0, sizeof(double) * 2 * nm, st);
+      if (e == cudaSuccess) {
+        for (int l = 1; l < nlev; ++l) launch_shift(A, off + l * nm, dim + l * nm, nm, shift[l], st);
+        launch_matrix_norm(A, off, dim, nm, mx, norm, st);
+        launch_invert(A, off, dim, n, mx, C, D, g.ainv, bad, st);
+        launch_matrix_norm(A, off, dim, nm, mx, norm + nm, st);
+        e = cudaGetLastError();
+      }
+      if (e == cudaSuccess) e = cudaMemcpyAsync(bad_h.data(), bad, sizeof(int) * n, cudaMemcpyDeviceToHost, st);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(norm_h.data(), norm, sizeof(double) * 2 * nm, cudaMemcpyDeviceToHost, st);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+      for (int r = 0; r < nm && e == cudaSuccess; ++r) {
+        const bool linear = !h.constants && dropped[r] == 0;
+        bool ok = 0x1p-24 * norm_h[r] * norm_h[nm + r] <= (!linear ? TEAM_COND_CONSTANT : sim->params.precision == CASIM_FP64 ? TEAM_COND_FP64 : TEAM_COND_MIXED);
+        for (int l = 0; l < nlev; ++l) ok = ok && !bad_h[l * nm + r];
+        if (ok || dropped[r] == 2) continue;
+        dropped[r] = linear ? 1 : 2;
+        drop_functions(h, r, linear ? 1 : 0);
+        again = true;
+      }
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(bad_h.data(), bad, sizeof(int) * n, cudaMemcpyDeviceToHost, st);
-    const cudaError_t e2 = cudaStreamSynchronize(st);
     cudaFree(tmp);
     CK(e);
-    CK(e2);
-    for (int b : bad_h)
-      if (b) h.coarse = false;
+    CK(up(g.z, h.z.data(), sizeof(float4) * h.z.size()));
+    if (std::count(dropped.begin(), dropped.end(), 2) == nm) h.coarse = false;
   }
   CK(cudaStreamSynchronize(st));
   h.halo = {};

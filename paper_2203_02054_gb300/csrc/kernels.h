@@ -33,6 +33,9 @@ static constexpr int TEAM_NT_F64 = 384;     //   one FP64 column of up to three 
 static constexpr int TEAM_LEVELS = 6;        //   inverses of the coarse matrix: for no springs,
 static constexpr float TEAM_SIGMA_1 = 1.0f / 1024;  //   springs per row of the next one (then a factor 4 each)
 static constexpr int TEAM_CONSTANTS_MAX = 4096; //   single MIXED robots up to this many rows: constants alone (see plan_team)
+static constexpr double TEAM_COND_FP64 = 0.125;  //   2^-24 |A_c| |A_c^-1| up to which the linear functions are
+static constexpr double TEAM_COND_MIXED = 0.25;  //   used, in FP64 and MIXED,
+static constexpr double TEAM_COND_CONSTANT = 1.0;  //   and the constants (see upload_team)
 static constexpr int INVERT_SLICE = 16384;  //   matrices inverted at once (a grid's z has at most 65,535)
 static constexpr size_t TEAM_SMEM_MAX = 216 * 1024;  //   dynamic shared memory
 static constexpr int PCG_CL_SIZE = 16;   // CTAs per cluster (non-portable size)
@@ -69,6 +72,8 @@ size_t team_words(bool fp64, int n_free, int parts, int robots, size_t& slot_off
 size_t team_smem(bool fp64, int rows, int r, int halo_max, int max_np, bool coarse, int max_width,
                  int& ainv_off, int& val_off, int& lcol_off);
 void launch_shift(double* A, const long long* off, const int* dim, int n_mat, double sigma, cudaStream_t st);
+void launch_matrix_norm(const double* A, const long long* off, const int* dim, int n_mat, int max_dim, double* norm,
+                        cudaStream_t st);
 void launch_invert(double* A, const long long* off, const int* dim, int n_mat, int max_dim, double* C, double* D,
                    float* out, int* bad, cudaStream_t st);
 template <typename T>

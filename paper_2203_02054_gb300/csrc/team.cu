@@ -1377,6 +1377,18 @@ __global__ void k_shift(double* A, const long long* off, const int* dim, double 
   if (i < n) A[off[blockIdx.y] + i * (n + 1)] += sigma;
 }
 
+// Largest absolute row sums (one warp to a row) into norm[r], which is zero before.
+__global__ void __launch_bounds__(256) k_matrix_norm(const double* A, const long long* off, const int* dim, double* norm) {
+  const int r = blockIdx.y, n = dim[r], i = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (i >= n) return;
+  double s = 0.0;
+  for (int j = threadIdx.x & 31; j < n; j += 32) s += fabs(A[off[r] + (long long)i * n + j]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  // (non-negative doubles order like their bits; a NaN ends above them)
+  if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned long long*>(norm + r), bits64(s));
+}
+
 // Calls f(first, count) for n_mat matrices (a batch has TEAM_LEVELS a robot) in
 // slices that fit a grid's y and z dimensions.
 template <typename F>
@@ -1387,6 +1399,13 @@ static void for_slices(int n_mat, F f) {
 void launch_shift(double* A, const long long* off, const int* dim, int n_mat, double sigma, cudaStream_t st) {
   for_slices(n_mat, [&](int s, int m) {
     k_shift<<<dim3((4 * TEAM_MAX_PARTS + 255) / 256, m), 256, 0, st>>>(A, off + s, dim + s, sigma);
+  });
+}
+
+void launch_matrix_norm(const double* A, const long long* off, const int* dim, int n_mat, int max_dim, double* norm,
+                        cudaStream_t st) {
+  for_slices(n_mat, [&](int s, int m) {
+    if (max_dim > 0) k_matrix_norm<<<dim3((max_dim + 7) / 8, m), 256, 0, st>>>(A, off + s, dim + s, norm + s);
   });
 }
 

@@ -1,0 +1,68 @@
+"""Bodies whose soft modes are far softer than their elements, where the coarse
+correction's FP32 inverse is not good enough: the solves still converge, within the
+iterations that they are given.  The residual of the returned positions, formed by
+the oracle's own system, is within the solver's tolerance and the rounding of that
+formula."""
+import numpy as np
+import pytest
+
+from paper_2203_02054_gb300 import casim, synth
+from oracle import global_step, local, loop
+
+pytestmark = pytest.mark.gpu
+
+FP64, MIXED = synth.PRECISION_FP64, synth.PRECISION_MIXED
+
+
+def _bar(nx, ny, nz, precision):
+    m = synth.config1_beam()
+    m.rest, m.tets, m.group, m.fixed = synth._voxel_kuhn(nx, ny, nz, 0.5,
+                                                         group_of_voxel=lambda i, j, k: 0 if k == nz - 1 else -1)
+    m.alpha = np.array([1.3])
+    m.precision, m.collision = precision, synth.COLLISION_OFF
+    return m
+
+
+def _check(m, Xi, X, tol):
+    """Residual at X of the global step that starts from Xi."""
+    p = loop.prepare(m.rest, m.tets, m.group, m.fixed)
+    P = local.local_step(Xi, p.tets, p.T_c, p.vol0, p.group, m.alpha, m.w_knots)[0]
+    A, b = global_step.assemble(p.tets, p.omega, P, p.n_verts, [], np.zeros((0, 3)), m.k_spring)
+    free = ~p.fixed.astype(bool)
+    F, C = A[free][:, free], A[free][:, ~free]
+    rhs = b[free] - C @ X[~free]
+    # (64 roundings of each term: about 20 of them in a row, the targets' and the right-hand side's)
+    size = abs(F) @ np.abs(X[free]) + abs(C) @ np.abs(X[~free]) + np.abs(b[free])
+    bound = tol * np.linalg.norm(rhs) + 64 * 2.0 ** -53 * np.linalg.norm(size)
+    assert np.linalg.norm(rhs - F @ X[free]) <= bound
+
+
+@pytest.mark.parametrize("precision,nx", [(FP64, 300), (FP64, 1500), (FP64, 2000), (MIXED, 1500), (MIXED, 3000)])
+def test_long_bodies_converge(precision, nx):
+    m = _bar(nx, 2, 2, precision)
+    sim = casim.Sim(m)
+    assert sim.stats().pcg_kernel == 5
+    X = m.rest
+    for _ in range(3):
+        Xi = X
+        sim.step(1)
+        assert sim.sync() == 0
+        X = sim.positions().astype(np.float64)
+        if precision == FP64:
+            _check(m, Xi, X, sim.params.pcg_tol)
+    sim.close()
+
+
+@pytest.mark.parametrize("precision", [FP64, MIXED])
+def test_a_long_body_in_a_batch(precision):
+    ms = [_bar(20, 4, 4, precision), _bar(2500, 2, 2, precision), _bar(31, 5, 4, precision)]
+    sim = casim.Sim(ms)
+    assert sim.stats().pcg_kernel == 5
+    sim.step(1)
+    assert sim.sync() == 0
+    X = sim.positions().astype(np.float64)
+    sim.close()
+    o = np.cumsum([0] + [m.n_verts for m in ms])
+    if precision == FP64:
+        for k, m in enumerate(ms):
+            _check(m, m.rest, X[o[k]:o[k + 1]], 1e-12)
