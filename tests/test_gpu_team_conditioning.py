@@ -66,3 +66,25 @@ def test_a_long_body_in_a_batch(precision):
     if precision == FP64:
         for k, m in enumerate(ms):
             _check(m, m.rest, X[o[k]:o[k + 1]], 1e-12)
+
+
+@pytest.mark.parametrize("thickness", [1e-3, 1e-4, 1e-5, 1e-6])
+@pytest.mark.parametrize("precision", [FP64, MIXED])
+def test_a_thin_layer_converges(precision, thickness):
+    """A layer of thin elements across the body: its far side hangs on a hundred
+    thousandth of an element's stiffness, a mode that no part's functions contain."""
+    m = _bar(40, 8, 8, precision)
+    layer = np.rint(m.rest[:, 0] / 0.5) >= 5
+    m.rest = m.rest.copy()
+    m.rest[layer, 0] -= 0.5 * (1.0 - thickness)
+    sim = casim.Sim(m)
+    assert sim.stats().pcg_kernel == 5
+    X = m.rest
+    for _ in range(4):
+        Xi = X
+        sim.step(1)
+        assert sim.sync() == 0
+        X = sim.positions().astype(np.float64)
+        if precision == FP64:
+            _check(m, Xi, X, sim.params.pcg_tol)
+    sim.close()
