@@ -79,9 +79,10 @@ typedef struct {
   double eps;               /* contact offset epsilon of Sec. II-C (length units)     */
   double pcg_tol;           /* stop when |r|_2 <= pcg_tol * |b|_2 (kernel 5 in FP64
                                with its two-level preconditioner: at 1/32 of it)      */
-  int32_t pcg_max_iter;     /* PCG iteration cap per outer iteration (an FP64 solve of
-                               kernel 5 that stalls goes on with Jacobi alone, to
-                               pcg_tol, and has as many again)                        */
+  int32_t pcg_max_iter;     /* PCG iteration cap per outer iteration (kernel 5, with a cap
+                               above 512: a solve that is not done after 512 with its
+                               two-level preconditioner goes on with Jacobi alone and
+                               has pcg_max_iter more)                                 */
   int32_t n_w_knots;        /* number of (strain, w) knots of R_omega, >= 1           */
   const double* w_knots;    /* host, 2*n_w_knots doubles (eps_i, w_i), eps ascending;
                                copied at casim_create                                 */

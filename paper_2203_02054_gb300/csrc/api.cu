@@ -485,6 +485,18 @@ Dev<T> make_dev(casim_sim* sim) {
   d.tm_lcol_off = sim->team.lcol_off;
   d.tm_cluster = sim->team.cluster;
   d.tm_coarse = sim->team.coarse ? 1 : 0;
+  // The coarse correction's FP32 rounding can keep a CG from finding modes that are
+  // softer than that rounding and outside the coarse space: a body that hangs on a
+  // layer of 1e-5 of an element's thickness did not converge in 6,000 FP64
+  // iterations, and takes 153 with Jacobi alone.  So a solve that is not done after
+  // so many starts its CG anew from where it is, with Jacobi alone and a cap of its
+  // own (thin layers: 610 to 1,120 iterations in all).  Solves that do converge with
+  // the correction took 230 at most (a body 3,000 voxels long).  A caller's lower cap
+  // ends the solve before.
+  const bool limited = sim->team.coarse && sim->params.pcg_max_iter > TEAM_COARSE_ITS;
+  d.tm_coarse_last = !sim->team.coarse ? -2 : limited ? TEAM_COARSE_ITS : 0x7FFFFFFE;
+  d.tm_cap = sim->params.pcg_max_iter;
+  if (limited) d.tm_cap += std::min(TEAM_COARSE_ITS, 0x7FFFFFFF - d.tm_cap);
   d.tm_levels = sim->team.levels;
   d.tm_halo_max = sim->team.halo_max;
   d.tm_halo = sim->tm.halo;

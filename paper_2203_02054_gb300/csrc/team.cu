@@ -65,14 +65,6 @@ static constexpr int TEAM_REFRESH = 8;  // iterations between fresh Z^T r sums
 // stop at 1/32 of the tolerance, so that finite differences of a run see no
 // more of that error than before (about a tenth more iterations).
 static constexpr double TEAM_STOP2_F64 = 1.0 / 1024.0;
-// An FP64 solve goes on without the coarse correction, as a Jacobi CG that starts
-// anew from where it is, once the squared residual has not fallen to a quarter in
-// this many iterations: the correction's FP32 rounding keeps a CG from finding
-// modes that are softer than that rounding and outside the coarse space.  A body
-// that hangs on a layer of a hundred thousandth of an element's thickness did not
-// converge in 6,000 iterations, takes 220 this way, and 153 with Jacobi alone.
-// Solves that do converge with the correction pause for 24 iterations at most.
-static constexpr int TEAM_STALL = 64;
 static constexpr int TEAM_MAXQ = 5;  // dot slots per lane of warp 0
 static_assert(32 * TEAM_MAXQ >= TEAM_MAX_PARTS, "a warp reads every slot of a team");
 
@@ -287,7 +279,6 @@ __device__ __forceinline__ S add_sums3(const S (*sa)[32], int q0, int q1) {
   for (int q = q0 + 1; q < q1; ++q) t = tree_add(t, sa[k][q]);
   return t;
 }
-__device__ __forceinline__ int high_word(double a) { return __double2hiint(a); }
 __device__ __forceinline__ DW acc_norm(DW a) { return dw_norm(a); }
 __device__ __forceinline__ double acc_norm(double a) { return a; }
 __device__ __forceinline__ DW shfl_at(DW v, int l) {
@@ -853,14 +844,9 @@ __global__ void __launch_bounds__(NTMAX, 1) k_pcg_team(const __grid_constant__ D
     float gs = 0.0f, gr = 0.0f;  // lane l < 12 of every warp: g(s) and g(r)
     int it = -1, f = CG_CONTINUE;
     bool lost = false;  // a wait gave up
-    int first = 0;      // the pass that starts the CG (a later one after a restart)
-    // FP64, warp 0: a squared residual below goal (high words) counts as progress;
-    // the last pass with any
-    constexpr int QUARTER = 2 << 20;
-    int goal = 0, moved = 0;
     for (;; ++it) {
       const unsigned e = (unsigned)it + 2u;  // epoch of this pass's u and round
-      const bool coarse = d.tm_coarse != 0 && (F32 || first == 0);
+      const bool coarse = it <= d.tm_coarse_last;
       A a[3];
       int which = 2;
       if (it < 0) {
@@ -1138,7 +1124,6 @@ __global__ void __launch_bounds__(NTMAX, 1) k_pcg_team(const __grid_constant__ D
             cg.bb = acc_to_f64(t0);
             cg.thr = tol2 * cg.bb;
             cg.rr = t1;
-            if constexpr (!F32) goal = high_word(t1) - QUARTER;
             if (t == 0) {
               s_es = acc_to_f64(t2);
               // a batch's energy is added up by the finalize launch: the
@@ -1148,17 +1133,7 @@ __global__ void __launch_bounds__(NTMAX, 1) k_pcg_team(const __grid_constant__ D
             f = (cg.bb > 0.0 && acc_to_f64(t1) > cg.thr) ? CG_CONTINUE : CG_DONE;
           } else {
             const A tot3[3] = {t0, t1, t2};
-            f = team_scalars(tot3, it == (F32 ? 0 : first), cg, ta, tb);
-            if constexpr (!F32)
-              if (coarse && f == CG_CONTINUE) {
-                // (squares order like their bits; on the integer pipes)
-                if (high_word(t2) < goal) {
-                  goal = high_word(t2) - QUARTER;
-                  moved = it;
-                } else if (it - moved == TEAM_STALL) {
-                  f = CG_RESTART;
-                }
-              }
+            f = team_scalars(tot3, it == 0 || it == d.tm_coarse_last + 1, cg, ta, tb);
           }
           if (f == CG_NONFINITE && c.me == 0 && t == 0) set_status(d.ctrl, ST_NONFINITE);
           if (t == 0) {
@@ -1186,12 +1161,6 @@ __global__ void __launch_bounds__(NTMAX, 1) k_pcg_team(const __grid_constant__ D
           }
           return x;
         };
-        if constexpr (!F32)
-          if (f == CG_RESTART) {
-            first = it + 1;
-            cg.thr = d.tol2 * cg.bb;
-            f = CG_CONTINUE;
-          }
         if (f != CG_CONTINUE) break;
         if (coarse) {
           if (which & 2) gr = shares(s_g[1]);
@@ -1203,7 +1172,7 @@ __global__ void __launch_bounds__(NTMAX, 1) k_pcg_team(const __grid_constant__ D
           __syncwarp();
         }
       }
-      if (it == (F32 ? 0 : first) + d.max_iter) {
+      if (it == d.tm_cap) {
         if (c.me == 0 && t == 0) set_status(d.ctrl, ST_PCG_MAXIT);
         break;
       }

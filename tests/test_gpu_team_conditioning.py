@@ -68,15 +68,20 @@ def test_a_long_body_in_a_batch(precision):
             _check(m, m.rest, X[o[k]:o[k + 1]], 1e-12)
 
 
-@pytest.mark.parametrize("thickness", [1e-3, 1e-4, 1e-5, 1e-6])
-@pytest.mark.parametrize("precision", [FP64, MIXED])
-def test_a_thin_layer_converges(precision, thickness):
-    """A layer of thin elements across the body: its far side hangs on a hundred
-    thousandth of an element's stiffness, a mode that no part's functions contain."""
-    m = _bar(40, 8, 8, precision)
+def _layered(nx, ny, nz, precision, thickness):
+    """A bar with a layer of thin elements across it: its far side hangs on that
+    fraction of an element's stiffness, a mode that no part's functions contain."""
+    m = _bar(nx, ny, nz, precision)
     layer = np.rint(m.rest[:, 0] / 0.5) >= 5
     m.rest = m.rest.copy()
     m.rest[layer, 0] -= 0.5 * (1.0 - thickness)
+    return m
+
+
+@pytest.mark.parametrize("thickness", [1e-3, 1e-4, 1e-5, 1e-6])
+@pytest.mark.parametrize("precision", [FP64, MIXED])
+def test_a_thin_layer_converges(precision, thickness):
+    m = _layered(40, 8, 8, precision, thickness)
     sim = casim.Sim(m)
     assert sim.stats().pcg_kernel == 5
     X = m.rest
@@ -87,4 +92,19 @@ def test_a_thin_layer_converges(precision, thickness):
         X = sim.positions().astype(np.float64)
         if precision == FP64:
             _check(m, Xi, X, sim.params.pcg_tol)
+    sim.close()
+
+
+# (in MIXED, with the linear functions: one row per thread, three)
+@pytest.mark.parametrize("precision,shape,thickness", [
+    (FP64, (40, 8, 8), 1e-5), (MIXED, (40, 8, 8), 1e-6), (MIXED, (150, 20, 20), 1e-5)])
+def test_thin_layers_in_batches_and_large_bodies(precision, shape, thickness):
+    ms = [_layered(*shape, precision, thickness)]
+    if shape[0] == 40:
+        ms.append(_bar(20, 4, 4, precision))
+    sim = casim.Sim(ms if len(ms) > 1 else ms[0])
+    assert sim.stats().pcg_kernel == 5
+    for _ in range(3):
+        sim.step(1)
+        assert sim.sync() == 0
     sim.close()
