@@ -497,6 +497,12 @@ Dev<T> make_dev(casim_sim* sim) {
   d.tm_coarse_last = !sim->team.coarse ? -2 : limited ? TEAM_COARSE_ITS : 0x7FFFFFFE;
   d.tm_cap = sim->params.pcg_max_iter;
   if (limited) d.tm_cap += std::min(TEAM_COARSE_ITS, 0x7FFFFFFF - d.tm_cap);
+  // Stiff springs make D^-1 the better preconditioner, and the correction, whose
+  // sigma is their mean, a hindrance.  CG iterations over four contact-bearing
+  // iterations with it and with Jacobi alone, by spring weight: 51,840 tets FP64 at
+  // 30 541 and 710, at 100 766 and 682, at 1,000 1,516 and 642; MIXED at 100 285 and
+  // 418, at 300 377 and 391, at 1,000 466 and 351 (1,219 and 187 for 6,480 tets).
+  d.tm_stiff = sim->params.k_spring > (sim->params.precision == CASIM_FP64 ? TEAM_STIFF_FP64 : TEAM_STIFF_MIXED);
   d.tm_levels = sim->team.levels;
   d.tm_halo_max = sim->team.halo_max;
   d.tm_halo = sim->tm.halo;

@@ -167,6 +167,7 @@ struct Dev {
   bool tm_cluster;           // the team is one thread-block cluster
   int tm_coarse;             // 1: two-level preconditioner
   int tm_coarse_last, tm_cap;  // the last CG pass with it (-2: none), the last pass
+  bool tm_stiff;             //   springs too stiff for it
   int tm_levels;             //   how many of its inverses are in use
   int tm_halo_max;           // longest halo (rows)
   const int* tm_halo;        // per part: the rows of other parts that its rows read, ascending

@@ -767,7 +767,9 @@ __global__ void __launch_bounds__(NTMAX, 1) k_pcg_team(const __grid_constant__ D
       int lvl = n_spr > 0 && d.tm_levels > 1 ? 1 : 0;
       for (float v = TEAM_SIGMA_1; lvl > 0 && lvl < d.tm_levels - 1 && v < sigma; v *= 4.0f) ++lvl;
       const float4* src = reinterpret_cast<const float4*>(d.tm_ainv + (size_t)lvl * d.tm_ainv_level + c.pt.ainv);
-      for (int k = t; k < nd; k += nt) reinterpret_cast<float4*>(ainv)[k] = src[k];
+      const bool stiff = n_spr > 0 && d.tm_stiff;  // zero: Jacobi alone (see make_dev)
+      for (int k = t; k < nd; k += nt)
+        reinterpret_cast<float4*>(ainv)[k] = stiff ? make_float4(0.0f, 0.0f, 0.0f, 0.0f) : src[k];
     }
     bool act[R];
     int width[R];

@@ -108,3 +108,26 @@ def test_thin_layers_in_batches_and_large_bodies(precision, shape, thickness):
         sim.step(1)
         assert sim.sync() == 0
     sim.close()
+
+
+@pytest.mark.parametrize("precision", [FP64, MIXED])
+@pytest.mark.parametrize("k_spring", [1e-3, 1.0, 1e3, 1e5])
+def test_spring_weights(precision, k_spring):
+    """The two-level preconditioner against Jacobi over contact-bearing iterations:
+    far from stiff springs it saves iterations, with them it costs few."""
+    its = []
+    for precond in (0, 1):
+        m = synth.small_finger(40, 8, 8, 5, seed=2, n_iters=1, precision=precision)
+        m.k_spring = k_spring
+        X0 = synth.perturbed_positions(m, 0.25, seed=7, dtype=np.float64 if precision == FP64 else np.float32)
+        sim = casim.Sim(m, pcg_precond=precond)
+        assert sim.stats().pcg_kernel == 5
+        sim.set_positions(X0)
+        sim.step(3)
+        assert sim.sync() == 0
+        h = sim.history()
+        assert all(r["n_springs"] > 0 for r in h)
+        its.append(sum(r["pcg_iters"] for r in h))
+        sim.close()
+    # (in FP64 the first stops at 1/32 of the second's tolerance, a tenth more iterations)
+    assert its[0] <= (1.25 if k_spring > 1 else 0.9) * its[1], its
