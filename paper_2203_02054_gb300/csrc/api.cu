@@ -749,7 +749,10 @@ void drop_functions(TeamHost& h, int r, int f0) {
 // larger norm, and failing that without a correction.  Bodies of 300 x 2 x 2
 // voxels reach 0.02 with the linear functions, of 1,200 0.18, and of 1,500 0.28,
 // where FP64 solves no longer converged with them, nor MIXED ones at 1.0 (3,000
-// voxels); constants alone reach 0.03 at 4,000.
+// voxels); constants alone reach 0.03 at 4,000.  FP64 robots of few rows go without
+// as well: their residuals can fall faster than g's FP32 rounding allows, and Jacobi
+// alone takes no more iterations (means, with and without: 13 and 8 at 8 to 15 rows,
+// 18 and 13 to 31, 22 and 17 to 63, 27 and 25 to 127, 29 and 28 to 255).
 int upload_team(casim_sim* sim) {
   TeamHost& h = sim->team;
   TeamDevice& g = sim->tm;
@@ -791,6 +794,11 @@ int upload_team(casim_sim* sim) {
     }
     std::vector<double> norm_h(2 * (size_t)nm);
     std::vector<int> dropped(nm, 0);  // 1: the linear functions, 2: all
+    for (int r = 0; r < nm; ++r)
+      if (sim->params.precision == CASIM_FP64 && sim->robot_row_h[r + 1] - sim->robot_row_h[r] < TEAM_COARSE_ROWS) {
+        dropped[r] = 2;
+        drop_functions(h, r, 0);
+      }
     cudaError_t e = up(off, off_h.data(), sizeof(long long) * n);
     if (e == cudaSuccess) e = up(dim, dim_h.data(), sizeof(int) * n);
     for (bool again = true; again && e == cudaSuccess;) {

@@ -268,7 +268,7 @@ struct DotAcc<double> {
   using type = double;
 };
 
-enum { CG_CONTINUE = 0, CG_DONE = 1, CG_NONFINITE = 2, CG_ABORT = 3 };
+enum { CG_CONTINUE = 0, CG_DONE = 1, CG_NONFINITE = 2, CG_ABORT = 3, CG_LOST = 4 };
 
 // CG scalars after the reduction of (gamma_k, delta_k, rr), by all of warp 0
 // (inputs read from lane 0, outputs in every lane).

@@ -34,6 +34,7 @@ static constexpr int TEAM_LEVELS = 6;        //   inverses of the coarse matrix:
 static constexpr float TEAM_SIGMA_1 = 1.0f / 1024;  //   springs per row of the next one (then a factor 4 each)
 static constexpr int TEAM_CONSTANTS_MAX = 4096; //   single MIXED robots up to this many rows: constants alone (see plan_team)
 static constexpr int TEAM_COARSE_ITS = 512;  //   CG iterations with the coarse correction (see make_dev)
+static constexpr int TEAM_COARSE_ROWS = 128;  //   FP64 robots with fewer rows do without it (see upload_team)
 static constexpr double TEAM_STIFF_FP64 = 50.0;  //   spring weights above which solves with springs do without
 static constexpr double TEAM_STIFF_MIXED = 200.0;  //   it (see make_dev)
 static constexpr double TEAM_COND_FP64 = 0.125;  //   2^-24 |A_c| |A_c^-1| up to which the linear functions are

@@ -685,6 +685,7 @@ __device__ __forceinline__ int team_scalars(const double (&t)[3], bool first, Cg
   const int lane = threadIdx.x & 31;
   if (!isfinite(t[0]) || !isfinite(t[1]) || !isfinite(t[2])) return CG_NONFINITE;
   double alpha;
+  bool lost = false;  // alpha is not positive (by the signs, beside the division)
   if (first) {
     alpha = t[0] / t[1];
     tb = 0.0;
@@ -692,8 +693,11 @@ __device__ __forceinline__ int team_scalars(const double (&t)[3], bool first, Cg
     cg.rr = t[2];
     if (t[2] <= cg.thr) return CG_DONE;
     // lane 0: gamma_k q / (delta_k q - gamma_k^2); lane 1: gamma_k / gamma_(k-1)
-    const double num = lane == 1 ? t[0] : t[0] * cg.q;
-    const double den = lane == 1 ? cg.gamma : fma(t[1], cg.q, -(t[0] * t[0]));
+    const double n0 = t[0] * cg.q, d0 = fma(t[1], cg.q, -(t[0] * t[0]));
+    const int hn = __double2hiint(n0), hd = __double2hiint(d0);
+    lost = (hn ^ hd) < 0 || hn == 0 || hd == 0;
+    const double num = lane == 1 ? t[0] : n0;
+    const double den = lane == 1 ? cg.gamma : d0;
     const double quo = num / den;
     tb = __shfl_sync(0xffffffffu, quo, 1);
     alpha = __shfl_sync(0xffffffffu, quo, 0);
@@ -701,7 +705,7 @@ __device__ __forceinline__ int team_scalars(const double (&t)[3], bool first, Cg
   ta = alpha;
   cg.gamma = t[0];
   cg.q = t[0] * alpha;
-  return CG_CONTINUE;
+  return lost ? CG_LOST : CG_CONTINUE;
 }
 
 // ------------------------------------------------------------- the solver
@@ -1136,6 +1140,18 @@ __global__ void __launch_bounds__(NTMAX, 1) k_pcg_team(const __grid_constant__ D
           } else {
             const A tot3[3] = {t0, t1, t2};
             f = team_scalars(tot3, it == 0 || it == d.tm_coarse_last + 1, cg, ta, tb);
+            // An FP64 residual that falls by 1e5 or more in a few iterations is less
+            // than the FP32 rounding that g has kept; the products with u then have any
+            // sign.  Such a pass moves nothing, and the CG starts anew with the next
+            // (there alpha is gamma / delta and beta 2^-60); g is formed anew before long.
+            if constexpr (!F32)
+              if (f == CG_LOST) {
+                f = CG_CONTINUE;
+                if (coarse) {
+                  ta = tb = T(0);
+                  cg.gamma = cg.q = 0x1p60 * t0;
+                }
+              }
           }
           if (f == CG_NONFINITE && c.me == 0 && t == 0) set_status(d.ctrl, ST_NONFINITE);
           if (t == 0) {
