@@ -268,6 +268,7 @@ struct DotAcc<double> {
   using type = double;
 };
 
+// (CG_LOST: the team PCG's step length is not positive)
 enum { CG_CONTINUE = 0, CG_DONE = 1, CG_NONFINITE = 2, CG_ABORT = 3, CG_LOST = 4 };
 
 // CG scalars after the reduction of (gamma_k, delta_k, rr), by all of warp 0
