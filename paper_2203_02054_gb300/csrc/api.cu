@@ -490,9 +490,9 @@ Dev<T> make_dev(casim_sim* sim) {
   // layer of 1e-5 of an element's thickness did not converge in 6,000 FP64
   // iterations, and takes 153 with Jacobi alone.  So a solve that is not done after
   // so many starts its CG anew from where it is, with Jacobi alone and a cap of its
-  // own (thin layers: 610 to 1,120 iterations in all).  Solves that do converge with
-  // the correction took 230 at most (a body 3,000 voxels long).  A caller's lower cap
-  // ends the solve before.
+  // own (thin layers: 510 to 1,120 iterations in all).  Solves of bodies without such
+  // layers took 230 at most with the correction (3,000 voxels long).  A caller's lower
+  // cap ends the solve before.
   const bool limited = sim->team.coarse && sim->params.pcg_max_iter > TEAM_COARSE_ITS;
   d.tm_coarse_last = !sim->team.coarse ? -2 : limited ? TEAM_COARSE_ITS : 0x7FFFFFFE;
   d.tm_cap = sim->params.pcg_max_iter;

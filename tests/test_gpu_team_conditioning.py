@@ -95,9 +95,10 @@ def test_a_thin_layer_converges(precision, thickness):
     sim.close()
 
 
-# (in MIXED, with the linear functions: one row per thread, three)
+# (FP64 in one cluster and in a batch; MIXED with the linear functions, one row per
+# thread in a batch and three)
 @pytest.mark.parametrize("precision,shape,thickness", [
-    (FP64, (40, 8, 8), 1e-5), (MIXED, (40, 8, 8), 1e-6), (MIXED, (150, 20, 20), 1e-5)])
+    (FP64, (16, 4, 4), 1e-7), (FP64, (40, 8, 8), 1e-5), (MIXED, (40, 8, 8), 1e-6), (MIXED, (150, 20, 20), 1e-5)])
 def test_thin_layers_in_batches_and_large_bodies(precision, shape, thickness):
     ms = [_layered(*shape, precision, thickness)]
     if shape[0] == 40:
